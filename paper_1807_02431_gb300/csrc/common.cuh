@@ -171,9 +171,36 @@ __device__ __forceinline__ void normals4_f32(const Philox4 &w, float xi[4]) {
 // ------------------------------------------------------------------------------------------------
 // Fixed-point accumulation: contributions converted with round-to-nearest; integer sums are exact
 // and independent of order, so results do not depend on the thread decomposition.
+// The conversion runs on the integer pipe: the significand of v 2^40 shifted to its place and rounded to
+// nearest even, the value of __double2ll_rn(v 2^40) for every |v| < 2^22.  As a compare, a multiply and a
+// conversion it took three instructions of the FP64 pipe, whose rate on sm_103a is 1/64 of the FP32 rate and
+// which bounds the FP64 kernels (22 beads, 256 replicas x 500 steps: 8.09 -> 7.07 ms; parameter gradient of 2,048
+// configurations of 100 beads, mixed: 535 -> 245 us).
+__device__ __forceinline__ long long fix_shift(unsigned long long m, int sh, bool neg) {
+  // m 2^sh rounded to an integer, sh <= 9 (double) or <= 38 (float); below 2^-54 every m < 2^53 rounds to 0
+  unsigned long long r;
+  if (sh >= 0) {
+    r = m << sh;
+  } else {
+    const int s = min(-sh, 54);
+    const unsigned long long rest = m << (64 - s);  // the dropped bits, from the top
+    r = m >> s;
+    r += (rest > 0x8000000000000000ull || (rest == 0x8000000000000000ull && (r & 1ull))) ? 1ull : 0ull;
+  }
+  return neg ? -(long long)r : (long long)r;
+}
 __device__ __forceinline__ long long to_fix(double v, int *err) {
-  if (!(fabs(v) < kFixLimit)) { *err |= kErrOverflow; return 0; }
-  return __double2ll_rn(v * kFixScale);
+  const int hi = __double2hiint(v), mag = hi & 0x7FFFFFFF;
+  if (mag >= 0x41500000) { *err |= kErrOverflow; return 0; }  // |v| >= 2^22, infinite or not a number
+  // (subnormal numbers get a leading one here and round to zero all the same)
+  const unsigned long long m = ((unsigned long long)((mag & 0xFFFFF) | 0x100000) << 32) | (unsigned int)__double2loint(v);
+  return fix_shift(m, (mag >> 20) - 1035, hi < 0);
+}
+// The same for a float: the value of to_fix((double)v).
+__device__ __forceinline__ long long to_fix(float v, int *err) {
+  const int b = __float_as_int(v), mag = b & 0x7FFFFFFF;
+  if (mag >= 0x4A800000) { *err |= kErrOverflow; return 0; }  // |v| >= 2^22, infinite or not a number
+  return fix_shift((unsigned long long)((mag & 0x7FFFFF) | 0x800000), (mag >> 23) - 110, b < 0);
 }
 // Mixed-path force accumulator: fixed point with 2^-32 units kept as two 32-bit words that are
 // summed separately with non-returning atomics (no carry between them; the 64-bit integer

@@ -79,12 +79,12 @@ __device__ __forceinline__ bool lj_param_terms(const V3<T> &d, const A &ai, cons
 struct ParamAcc {
   long long *G;
   __device__ __forceinline__ void add(int k, double v, int *err) const { fix_add(&G[k], to_fix(v, err)); }
-  __device__ __forceinline__ void add(int k, float v, int *err) const { fix_add(&G[k], to_fix((double)v, err)); }
+  __device__ __forceinline__ void add(int k, float v, int *err) const { fix_add(&G[k], to_fix(v, err)); }
 };
 struct ParamTangent {
   long long *G;
   __device__ __forceinline__ void add(int k, Dual v, int *err) const { fix_add(&G[k], to_fix(v.d, err)); }
-  __device__ __forceinline__ void add(int k, DualF v, int *err) const { fix_add(&G[k], to_fix((double)v.d, err)); }
+  __device__ __forceinline__ void add(int k, DualF v, int *err) const { fix_add(&G[k], to_fix(v.d, err)); }
 };
 
 // dV/d theta of one configuration by the whole block; qd(i, j) gives q_i - q_j in type T.

@@ -1,0 +1,44 @@
+"""The integer conversions to the 2^-40 fixed point, through the forces of one bond whose arithmetic is
+exact, and the column sums of the parameter gradient at the edges of their row blocks."""
+import numpy as np
+import pytest
+
+from paper_1807_02431_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_1807_02431_gb300 import binding
+
+    binding.load()
+    return binding
+
+
+def _bond(k, x, r0):
+    """Two atoms x apart on the first axis, one bond (k, r0) and nothing else."""
+    s = W.System(name="bond", n_atoms=2, dim=3, potential=W.POT_FORCE_FIELD, mass=np.ones(2), kT=1.0, gamma=1.0, dt=1e-3,
+                 sigma=np.full(2, 0.3), epsilon=np.zeros(2), charge=np.zeros(2), excl=np.array([[0, 1]], np.int32),
+                 bonds=np.array([[0, 1]], np.int32), bond_k=np.array([k]), bond_r0=np.array([r0]),
+                 cv_kind=W.CV_COM_DISTANCE, cv_params=(1.0,), groups=[[0], [1]])
+    s.q0, s.p0 = np.array([[0.0, 0, 0], [x, 0, 0]]), np.zeros((2, 3))
+    return s
+
+
+@pytest.mark.parametrize("sign", [1, -1])
+@pytest.mark.parametrize("e", [-60, -43, -42, -41, -40, -39, -30, -20, -10, 0, 11, 12, 13, 20, 21])
+def test_fp64_fixed_point_of_a_force(B, e, sign):
+    """Force k (r - r0) with every factor a few bits long, so that it is exact before the conversion: the
+    result is the nearest multiple of 2^-40 (ties to even), whatever its size below 2^22."""
+    import torch
+
+    for m in (1.0, 1.5, 1.25, 1.75, 1.0 + 2.0 ** -12):
+        x, r0 = (2.0, 1.0) if sign > 0 else (1.0, 2.0)
+        k = m * 2.0 ** e  # force on atom 0 towards atom 1 when stretched: k (r - r0) = +-k
+        sysh = B.grp_create_system(_bond(k, x, r0), B.GRP_FP64)
+        q = torch.tensor([[[0.0, 0, 0], [x, 0, 0]]], dtype=torch.float64, device="cuda")
+        f = torch.empty_like(q)
+        B.grp_energy_forces(sysh, 1, q, None, f)
+        want = sign * np.rint(k * 2.0 ** 40) * 2.0 ** -40
+        assert f[0, 0, 0].item() == want and f[0, 1, 0].item() == -want
