@@ -429,7 +429,7 @@ grp_status grp_set_params(grp_system *s, const double *d_theta, void *stream);
 /* For B configurations d_q (device [B][n][dim] FP64) and weights d_w (device [B], NULL = all 1):
  *   d_energy     (optional, device [B])        V(q_b), unweighted;
  *   d_grad_q     (optional, device [B][n][dim]) w_b dV/dq (q_b) = -w_b F(q_b);
- *   d_grad_theta (optional, device [n_theta])   sum_b w_b dV/d theta (q_b), summed in order of b.
+ *   d_grad_theta (optional, device [n_theta])   sum_b w_b dV/d theta (q_b), summed in a fixed order.
  * This is the vector-Jacobian product of the map q -> (V(q_b))_b for the cotangent w, as reverse-
  * mode differentiation needs it.  Computed in the system's precision (the mixed path: FP32 terms,
  * fixed-point sums).  Synchronises `stream`. */

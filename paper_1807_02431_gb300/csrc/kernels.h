@@ -165,7 +165,7 @@ struct AdjArgs {
 };
 size_t adjoint_smem_bytes(const SysDev &S, int n_terms, int ck);
 cudaError_t launch_adjoint(const AdjArgs &a, int n_rep, cudaStream_t st);
-// out[t] = sum_b partial[b][t] in order of b.
+// out[t] = sum_b partial[b][t] in a fixed order.
 cudaError_t launch_column_sum(const double *partial, int rows, int cols, double *out, cudaStream_t st);
 
 }  // namespace grp

@@ -42,3 +42,25 @@ def test_fp64_fixed_point_of_a_force(B, e, sign):
         B.grp_energy_forces(sysh, 1, q, None, f)
         want = sign * np.rint(k * 2.0 ** 40) * 2.0 ** -40
         assert f[0, 0, 0].item() == want and f[0, 1, 0].item() == -want
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("n_conf", [1, 2, 63, 64, 65, 127, 129, 200])
+def test_param_gradient_sums(B, n_conf, prec):
+    """The summed parameter gradient against the single configurations' added up in extended precision: sums of
+    n terms in another order differ by at most n eps of the sum of magnitudes."""
+    import torch
+
+    s = W.chain(22)
+    sysh = B.grp_create_system(s, B.GRP_FP64 if prec == "fp64" else B.GRP_MIXED)
+    q = torch.from_numpy(W.replica_states(s, n_conf, seed=5, spread=0.01)[0]).cuda()
+    n = B.grp_param_count(sysh)
+    one, tot = (torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(2))
+    B.grp_energy_grad(sysh, n_conf, q, None, None, None, tot)
+    want, mag = np.zeros(n, np.longdouble), np.zeros(n)
+    for b in range(n_conf):
+        B.grp_energy_grad(sysh, 1, q[b:b + 1].contiguous(), None, None, None, one)
+        v = one.cpu().numpy()
+        want += v
+        mag += np.abs(v)
+    assert np.all(np.abs(tot.cpu().numpy() - want) <= n_conf * 2.0 ** -53 * mag)
