@@ -1014,6 +1014,9 @@ extern "C" grp_status grp_batch_create(grp_replicas *const *runs, int32_t n_runs
     return runs[x.x]->sys->dev.n > runs[y.x]->sys->dev.n;
   });
   b->threads = std::min(512, b->threads);
+  bool items = true;
+  for (int i = 0; i < n_runs; ++i) items = items && !runs[i]->sys->dev.tiled;
+  if (items) b->threads = batch_threads(b->precision, b->threads, b->smem, (int)units.size());
   b->n_units = (int)units.size();
   b->n_branch_units = (int)bunits.size();
   b->n_gr_units = (int)gunits.size();

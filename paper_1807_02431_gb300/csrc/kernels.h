@@ -37,6 +37,8 @@ struct SegArgs {
   double h, c1;              // dt/2 and exp(-gamma dt)
 };
 
+constexpr int kMaxThreadChoices = 4;
+
 // Launch configuration chosen per system (threads per replica block).
 struct SegConfig {
   int threads;
@@ -44,12 +46,18 @@ struct SegConfig {
   int pairs_in_smem;
   int noise_batch;
   int lean;
+  // smaller blocks for many replicas (item-table systems): choice[0] = threads, and how many blocks of each size
+  // the device holds at once
+  int n_choices;
+  int choice[kMaxThreadChoices], slots[kMaxThreadChoices];
 };
 
 // Largest dynamic shared memory of one block on sm_103a.
 constexpr size_t kMaxSmem = 227 * 1024;
 
 SegConfig segment_config(const SysDev &S, int threads_hint);
+// Block size of the batched kernel for `units` replicas of item-table systems that take up to `threads` each.
+int batch_threads(int precision, int threads, size_t smem, int units);
 // The noise amplitude of every atom in FP64 and FP32 (the system's tables for lean replica states).
 cudaError_t launch_noise_sd(const SysDev &S, double c1, double *sd_d, float *sd_f, cudaStream_t st);
 cudaError_t launch_segment(const SegArgs &a, const SegConfig &cfg, cudaStream_t st);

@@ -800,6 +800,72 @@ static size_t ff_smem_bytes(const SysDev &S, int pairs_in_smem, int noise_batch,
   return b;
 }
 
+// The segment kernel of a system for blocks of `threads`.
+template <class P>
+static auto ff_kernel(const SysDev &S, int threads) {
+  const int mode = S.use_list ? kModeList : (S.tiled ? kModeTiles : kModeItems);
+  const bool small = threads <= 320;
+  // tiles are taken only without a cutoff, so never with the reaction field; implicit solvent only on
+  // the item table (and never with a cutoff)
+  const bool rf = S.coulomb_rf == 1, gb = S.gb != 0, con = S.n_cons > 0, pme = S.coulomb_rf == 2;
+  return mode == kModeItems
+                  ? (pme  ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 4> : ff_segment_kernel<P, 512, 1, kModeItems, 4>)
+                     : con ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 3> : ff_segment_kernel<P, 512, 1, kModeItems, 3>)
+                     : gb ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 2> : ff_segment_kernel<P, 512, 1, kModeItems, 2>)
+                     : rf ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 1> : ff_segment_kernel<P, 512, 1, kModeItems, 1>)
+                          : (small ? ff_segment_kernel<P, 320, 2, kModeItems, 0> : ff_segment_kernel<P, 512, 1, kModeItems, 0>))
+            : mode == kModeTiles
+                  ? (small ? ff_segment_kernel<P, 320, 2, kModeTiles, 0> : ff_segment_kernel<P, 512, 1, kModeTiles, 0>)
+                  : pme ? ff_segment_kernel<P, 512, 1, kModeList, 4>  // periodic (the mesh's registers)
+                  : (rf ? (small ? ff_segment_kernel<P, 320, 2, kModeList, 1> : ff_segment_kernel<P, 512, 1, kModeList, 1>)
+                     : (gb && con) ? (small ? ff_segment_kernel<P, 320, 2, kModeList, 5> : ff_segment_kernel<P, 512, 1, kModeList, 5>)
+                     : gb ? (small ? ff_segment_kernel<P, 320, 2, kModeList, 2> : ff_segment_kernel<P, 512, 1, kModeList, 2>)
+                     : con ? (small ? ff_segment_kernel<P, 320, 2, kModeList, 3> : ff_segment_kernel<P, 512, 1, kModeList, 3>)
+                          : (small ? ff_segment_kernel<P, 320, 2, kModeList, 0> : ff_segment_kernel<P, 512, 1, kModeList, 0>));
+}
+
+// Blocks of the kernel that the device holds at once (0: unknown).
+template <class K>
+static int resident_blocks(K kern, int threads, size_t smem) {
+  int dev = 0, sms = 0, per_sm = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return sms * per_sm;
+}
+
+// Block sizes of item-table systems.  One thread per item is the shortest step while every replica has a place on
+// the chip; a step is a chain of latencies, so with more replicas smaller blocks, of which more are resident, do
+// more steps per second.  Candidates from the default downwards, of which a launch takes the largest whose
+// blocks are all resident, or else the last: 512, 320, 192, 160 threads, and 64, 32 for systems of up to 128 items
+// (7 to 10 beads).  us per 100 steps, default -> chosen (mixed): 40 beads 256 replicas 466 -> 375 (512 -> 320
+// threads), 1,024 replicas 1,614 -> 1,185 (160); 60 beads 256 replicas 855 -> 756; 22 beads 400 replicas 303 -> 231
+// (192), 1,024 replicas 625 -> 485 (160); 24 atoms with constraints, 512 replicas 1,458 -> 856; solvated 22 beads,
+// 512 replicas 826 -> 709; FP64 22 beads, 1,024 replicas 6,470 -> 5,220; batch of 2,048 alkanes of 7 beads 1,277 ->
+// 989 (32).  Sizes between (96, 128, 224, 256) were within 5 % or slower.  The particle mesh keeps its 320.
+static int thread_candidates(int threads, int out[kMaxThreadChoices]) {
+  static const int kLarge[] = {320, 192, 160}, kSmall[] = {64, 32};
+  int n = 0;
+  out[n++] = threads;
+  if (threads <= 128) {
+    for (int c : kSmall)
+      if (c < threads) out[n++] = c;
+  } else {
+    for (int c : kLarge)
+      if (c < threads) out[n++] = c;
+  }
+  return n;
+}
+static int choose_threads(const int *threads, const int *slots, int n, int units) {
+  for (int t = 0; t < n; ++t)
+    if (units <= slots[t]) return threads[t];
+  return threads[n - 1];
+}
+
 SegConfig segment_config(const SysDev &S, int threads_hint) {
   SegConfig c{};
   if (S.potential == GRP_POT_DOUBLE_WELL_2D) {
@@ -840,34 +906,38 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
   }
   c.pairs_in_smem = ff_smem_bytes(S, 1, nb, c.lean) <= 160 * 1024 ? 1 : 0;
   c.smem = ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean);
+  c.n_choices = 1;
+  c.choice[0] = c.threads;
+  if (!S.tiled && S.coulomb_rf != 2 && threads_hint <= 0 && c.smem <= kMaxSmem) {
+    c.n_choices = thread_candidates(c.threads, c.choice);
+    for (int t = 0; t < c.n_choices; ++t) {
+      c.slots[t] = S.precision == GRP_FP64 ? resident_blocks(ff_kernel<PathF64>(S, c.choice[t]), c.choice[t], c.smem)
+                                           : resident_blocks(ff_kernel<PathMixed>(S, c.choice[t]), c.choice[t], c.smem);
+      if (c.slots[t] == 0) c.n_choices = 1;  // nothing known: the default
+    }
+  }
   return c;
+}
+
+int batch_threads(int precision, int threads, size_t smem, int units) {
+  int cand[kMaxThreadChoices], slots[kMaxThreadChoices];
+  const int n = thread_candidates(threads, cand);
+  for (int t = 0; t < n; ++t) {
+    slots[t] = precision == GRP_FP64 ? resident_blocks(ff_segment_batch_kernel<PathF64>, cand[t], smem)
+                                     : resident_blocks(ff_segment_batch_kernel<PathMixed>, cand[t], smem);
+    if (slots[t] == 0) return threads;
+  }
+  return choose_threads(cand, slots, n, units);
 }
 
 template <class P>
 static cudaError_t launch_ff_p(const SegArgs &a, const SegConfig &c, cudaStream_t st) {
-  if (c.threads < 32 || c.threads > 512 || c.threads % 32) return cudaErrorInvalidValue;
-  const int mode = a.S.use_list ? kModeList : (a.S.tiled ? kModeTiles : kModeItems);
-  const bool small = c.threads <= 320;
-  // tiles are taken only without a cutoff, so never with the reaction field; implicit solvent only on
-  // the item table (and never with a cutoff)
-  const bool rf = a.S.coulomb_rf == 1, gb = a.S.gb != 0, con = a.S.n_cons > 0, pme = a.S.coulomb_rf == 2;
-  auto kern = mode == kModeItems
-                  ? (pme  ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 4> : ff_segment_kernel<P, 512, 1, kModeItems, 4>)
-                     : con ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 3> : ff_segment_kernel<P, 512, 1, kModeItems, 3>)
-                     : gb ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 2> : ff_segment_kernel<P, 512, 1, kModeItems, 2>)
-                     : rf ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 1> : ff_segment_kernel<P, 512, 1, kModeItems, 1>)
-                          : (small ? ff_segment_kernel<P, 320, 2, kModeItems, 0> : ff_segment_kernel<P, 512, 1, kModeItems, 0>))
-            : mode == kModeTiles
-                  ? (small ? ff_segment_kernel<P, 320, 2, kModeTiles, 0> : ff_segment_kernel<P, 512, 1, kModeTiles, 0>)
-                  : pme ? ff_segment_kernel<P, 512, 1, kModeList, 4>  // periodic (the mesh's registers)
-                  : (rf ? (small ? ff_segment_kernel<P, 320, 2, kModeList, 1> : ff_segment_kernel<P, 512, 1, kModeList, 1>)
-                     : (gb && con) ? (small ? ff_segment_kernel<P, 320, 2, kModeList, 5> : ff_segment_kernel<P, 512, 1, kModeList, 5>)
-                     : gb ? (small ? ff_segment_kernel<P, 320, 2, kModeList, 2> : ff_segment_kernel<P, 512, 1, kModeList, 2>)
-                     : con ? (small ? ff_segment_kernel<P, 320, 2, kModeList, 3> : ff_segment_kernel<P, 512, 1, kModeList, 3>)
-                          : (small ? ff_segment_kernel<P, 320, 2, kModeList, 0> : ff_segment_kernel<P, 512, 1, kModeList, 0>));
+  const int threads = c.n_choices > 1 ? choose_threads(c.choice, c.slots, c.n_choices, a.n_active) : c.threads;
+  if (threads < 32 || threads > 512 || threads % 32) return cudaErrorInvalidValue;
+  auto kern = ff_kernel<P>(a.S, threads);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);
   if (e != cudaSuccess) return e;
-  kern<<<a.n_active, c.threads, c.smem, st>>>(a);
+  kern<<<a.n_active, threads, c.smem, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -53,3 +53,39 @@ def test_double_well_groups(B, oracle_mod, R, k):
         B.grp_step_k(part, k, 5)
         qs, ps, accs, _ = B.grp_get_state(part)
         assert np.array_equal(q[lo:], qs) and np.array_equal(p[lo:], ps) and np.array_equal(acc[lo:], accs)
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("make", ["chain10", "chain22", "chain40", "chain_h", "solvated"])
+def test_block_sizes_give_the_same_bits(B, make, prec):
+    """Large sets run with smaller blocks than small ones: the fixed-point sums do not depend on the
+    decomposition, so the first replicas are those of a small set bit for bit."""
+    s = {"chain10": lambda: W.chain(10), "chain22": lambda: W.chain(22), "chain40": lambda: W.chain(40),
+         "chain_h": lambda: W.chain_h(12), "solvated": lambda: W.solvated(W.chain(14))}[make]()
+    R, small, k = 2600, 5, 12
+    q0, p0 = W.replica_states(s, R, seed=9, spread=0.002)
+    sysh = B.grp_create_system(s, B.GRP_FP64 if prec == "fp64" else B.GRP_MIXED)
+    out = []
+    for n in (small, 320, 470, R):
+        rep = B.grp_init_replicas(sysh, n, SEED, q0[:n], p0[:n], per_replica=True)
+        B.grp_step_k(rep, k, 4)
+        q, p, acc, _ = B.grp_get_state(rep)
+        out.append((q[:small], p[:small], acc[:small]))
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n_runs", [2, 40, 130])
+def test_batched_block_sizes_give_the_same_bits(B, n_runs):
+    """Batches of small systems: up to 130 x 20 = 2,600 units, against the runs alone."""
+    s, R, k = W.alkane(), 20, 30
+    sysh = B.grp_create_system(s, B.GRP_MIXED)
+    q0, p0 = W.replica_states(s, R, seed=2, spread=0.002)
+    runs = [B.grp_init_replicas(sysh, R, SEED + i, q0, p0, per_replica=True) for i in range(n_runs)]
+    B.grp_batch_step_k(B.grp_batch_create(runs), k, 5)
+    for i in (0, n_runs - 1):
+        alone = B.grp_init_replicas(sysh, R, SEED + i, q0, p0, per_replica=True)
+        B.grp_step_k(alone, k, 5)
+        for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(runs[i])[:3]):
+            assert np.array_equal(a, b)
