@@ -154,17 +154,40 @@ __device__ __forceinline__ void param_pass(const SysDev &S, const A *atom, const
 }
 
 // One block per configuration b; G[2n + n_terms] fixed-point accumulators in shared memory.
-template <class T, class A, class A4T>
-__global__ void __launch_bounds__(256) param_grad_kernel(SysDev S, const A *atom, const A4T *term, int n_terms,
-                                                         const double *q, const double *w, double *grad_q,
+// kStaged (mixed path, where it fits): the positions wait in shared memory as double-single numbers and their
+// differences are formed in FP32.  An FP64 subtraction and conversion per coordinate and pair cost six instructions of
+// the FP64 pipe (1/64 of the FP32 rate) and three 8-byte loads per atom from memory: energies and gradients of
+// 2,048 configurations of 100 beads 396 -> 285 us.
+template <class T, class A, class A4T, bool kStaged>
+__global__ void __launch_bounds__(256) param_grad_kernel(const __grid_constant__ SysDev S, const A *atom, const A4T *term,
+                                                         int n_terms, const double *q, const double *w, double *grad_q,
                                                          double *partial, int *errp) {
   extern __shared__ __align__(16) long long G[];
   const int n = S.n, nt = 2 * n + n_terms, b = blockIdx.x;
   const double *qb = q + (size_t)b * S.nd;
   for (int i = threadIdx.x; i < nt; i += blockDim.x) G[i] = 0;
+  float4 *hi = reinterpret_cast<float4 *>(G + ((nt + 1) & ~1)), *lo = hi + n;
+  if constexpr (kStaged)
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const ds x = ds_from_double(qb[3 * i]), y = ds_from_double(qb[3 * i + 1]), v = ds_from_double(qb[3 * i + 2]);
+      hi[i] = make_float4(x.hi, y.hi, v.hi, 0.f);
+      lo[i] = make_float4(x.lo, y.lo, v.lo, 0.f);
+    }
   __syncthreads();
   int err = 0;
-  param_pass<T>(S, atom, term, [&](int i, int j) { return qdiff<T>(qb, i, j); }, ParamAcc{G}, &err);
+  if constexpr (kStaged) {
+    auto sub = [](float ah, float al, float bh, float bl) {
+      const float s = __fsub_rn(ah, bh), bp = __fsub_rn(s, ah);
+      const float e = __fadd_rn(__fsub_rn(ah, __fsub_rn(s, bp)), __fsub_rn(-bh, bp));  // TwoSum(a, -b)
+      return __fadd_rn(s, __fadd_rn(e, __fsub_rn(al, bl)));
+    };
+    param_pass<T>(S, atom, term, [&](int i, int j) {
+      const float4 a = hi[i], b = hi[j], c = lo[i], d = lo[j];
+      return V3<T>{sub(a.x, c.x, b.x, d.x), sub(a.y, c.y, b.y, d.y), sub(a.z, c.z, b.z, d.z)};
+    }, ParamAcc{G}, &err);
+  } else {
+    param_pass<T>(S, atom, term, [&](int i, int j) { return qdiff<T>(qb, i, j); }, ParamAcc{G}, &err);
+  }
   __syncthreads();
   const double wb = w ? w[b] : 1.0;
   for (int i = threadIdx.x; i < nt; i += blockDim.x) partial[(size_t)b * nt + i] = wb * ((double)G[i] * kFixInv);
@@ -181,13 +204,17 @@ cudaError_t launch_param_grad(const SysDev &S, int n_terms, int n_conf, const do
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   cudaError_t e;
   if (S.precision == GRP_FP64) {
-    auto k = param_grad_kernel<double, double4, double4>;
+    auto k = param_grad_kernel<double, double4, double4, false>;
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
     k<<<n_conf, 256, smem, st>>>(S, S.atom_d, S.term_d, n_terms, q, w, grad_q, partial, err);
   } else {
-    auto k = param_grad_kernel<float, float4, float4>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    k<<<n_conf, 256, smem, st>>>(S, S.atom_f, S.term_f, n_terms, q, w, grad_q, partial, err);
+    // staged while two blocks share an SM
+    const size_t staged = smem + 8 + (size_t)S.n * 32;
+    const bool fits = staged <= 113 * 1024;
+    auto k = fits ? param_grad_kernel<float, float4, float4, true> : param_grad_kernel<float, float4, float4, false>;
+    const size_t bytes = fits ? staged : smem;
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    k<<<n_conf, 256, bytes, st>>>(S, S.atom_f, S.term_f, n_terms, q, w, grad_q, partial, err);
   }
   return cudaGetLastError();
 }

@@ -64,3 +64,28 @@ def test_param_gradient_sums(B, n_conf, prec):
         want += v
         mag += np.abs(v)
     assert np.all(np.abs(tot.cpu().numpy() - want) <= n_conf * 2.0 ** -53 * mag)
+
+
+@pytest.mark.parametrize("n", [22, 33, 64, 100])
+def test_param_gradient_against_autograd(B, n):
+    """Mixed-path parameter gradients (positions staged as double-single numbers) far from the origin, where an FP32
+    position would have lost the difference: against 64-bit automatic differentiation of the Lennard-Jones and
+    torsion terms.  A pair's term is some twenty FP32 operations (1e-6 of its size); the sums have no rounding."""
+    import torch
+
+    s = W.chain(n)
+    q = W.replica_states(s, 3, seed=8, spread=0.01)[0] + np.array([40.0, -25.0, 60.0])
+    sysh = B.grp_create_system(s, B.GRP_MIXED)
+    got = torch.empty(B.grp_param_count(sysh), dtype=torch.float64, device="cuda")
+    B.grp_energy_grad(sysh, 3, torch.from_numpy(q).cuda(), None, None, None, got)
+    sig, eps = (torch.tensor(x, requires_grad=True) for x in (s.sigma, s.epsilon))
+    keep = np.ones((n, n), bool)
+    keep[s.excl[:, 0], s.excl[:, 1]] = keep[s.excl[:, 1], s.excl[:, 0]] = False
+    i, j = (torch.from_numpy(x) for x in np.nonzero(np.triu(keep, 1)))
+    x = torch.from_numpy(q)
+    s6 = (0.25 * (sig[i] + sig[j]) ** 2 / ((x[:, i] - x[:, j]) ** 2).sum(-1)) ** 3
+    e = 4.0 * torch.sqrt(eps[i] * eps[j]) * (s6 * s6 - s6)
+    size = [torch.autograd.grad(e.abs().sum(), v, retain_graph=True)[0].abs().numpy().max() for v in (sig, eps)]
+    want = [v.numpy() for v in torch.autograd.grad(e.sum(), (sig, eps))]
+    for w, g, m in zip(want, (got[:n].cpu().numpy(), got[n:2 * n].cpu().numpy()), size):
+        assert np.abs(g - w).max() <= 1e-6 * m
