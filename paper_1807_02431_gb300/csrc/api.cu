@@ -340,6 +340,7 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
       excl[(size_t)i * n + j] = excl[(size_t)j * n + i] = 1;
     }
     D.cutoff2 = d->cutoff > 0 ? d->cutoff * d->cutoff : 0.0;
+    D.cutoff2_f = (float)D.cutoff2;
     if (d->coulomb_mode == GRP_COULOMB_REACTION_FIELD) {
       if (!(d->cutoff > 0)) { grp_destroy_system(s); return fail(GRP_EINVAL, "the reaction field needs cutoff > 0"); }
       if (!(d->rf_dielectric == 0.0 || d->rf_dielectric >= 1.0)) {
@@ -444,6 +445,61 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
       bij.swap(bij2);
       bd.swap(bd2);
       bf.swap(bf2);
+    }
+    // Large systems on the mixed path, in vacuum: neighbour rows (rows.cuh), from as many tiles as keep sixteen
+    // warps busy with whole tiles
+    D.use_rows = D.use_list && d->precision == GRP_MIXED && !d->gb_radius && D.coulomb_rf != 2 && n >= kRowsMinAtoms;
+    if (D.use_rows) {
+      // Static rows of partners (rows.cuh): each pair on the row of the atom whose row is shorter so far (the
+      // first atom's when equal); place [t / 4][i][t % 4] for partner t of atom i, 0xFFFF past the atom's last
+      struct StaticRows {
+        int blocks = 0;
+        std::vector<int> tile_rows;
+        std::vector<size_t> place;  // of each pair
+        std::vector<uint16_t> partner;
+      };
+      auto static_rows = [&](const std::vector<int2> &ij) {
+        StaticRows out;
+        const int nt = (n + 31) / 32;
+        std::vector<int> len(n, 0);
+        std::vector<int> other;
+        for (const int2 &p : ij) {
+          const bool swap = len[p.y] < len[p.x];
+          const int i = swap ? p.y : p.x, t = len[i]++;
+          out.place.push_back(((size_t)(t / 4) * n + i) * 4 + t % 4);
+          other.push_back(swap ? p.x : p.y);
+        }
+        out.tile_rows.assign(nt, 0);
+        for (int i = 0; i < n; ++i) out.tile_rows[i / 32] = std::max(out.tile_rows[i / 32], len[i]);
+        for (int v : out.tile_rows) out.blocks = std::max(out.blocks, (v + 3) / 4);
+        out.partner.assign((size_t)out.blocks * n * 4, 0xFFFF);
+        for (size_t u = 0; u < ij.size(); ++u) out.partner[out.place[u]] = (uint16_t)other[u];
+        return out;
+      };
+      std::vector<int2> soft;
+      std::vector<int> index, stiff;
+      for (int b = 0; b < d->n_bonds; ++b) {
+        if (bf[b].x >= kSoftBond) { stiff.push_back(b); continue; }
+        soft.push_back(bij[b]);
+        index.push_back(b);
+      }
+      const StaticRows sr = static_rows(soft);
+      std::vector<float2> kf(sr.partner.size(), make_float2(0.f, 0.f));
+      for (size_t u = 0; u < soft.size(); ++u) kf[sr.place[u]] = bf[index[u]];
+      UP(sr.tile_rows.data(), sr.tile_rows.size(), &D.spring_rows);
+      UP(reinterpret_cast<const ushort4 *>(sr.partner.data()), sr.partner.size() / 4, &D.spring_j);
+      UP(reinterpret_cast<const float4 *>(kf.data()), kf.size() / 2, &D.spring_f);
+      D.n_stiff = (int)stiff.size();
+      UP(stiff.data(), stiff.size(), &D.stiff);
+      // a pair is on the row of its lower atom when the sum of the two is odd, of the higher when it is even, so
+      // that every atom has about half of its neighbours on its row
+      const int nt = D.n_tiles;
+      std::vector<uint32_t> rmask((size_t)nt * nt * 32, 0);
+      for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j)
+          if (i != j && !excl[(size_t)i * n + j] && (((i + j) & 1) ? i < j : i > j))
+            rmask[((size_t)(i / 32) * nt + j / 32) * 32 + i % 32] |= 1u << (j % 32);
+      UP(rmask.data(), rmask.size(), &D.row_masks);
     }
     D.n_bonds = d->n_bonds;
     UP(bij.data(), bij.size(), &D.bond_ij);
@@ -800,7 +856,8 @@ extern "C" grp_status grp_init_replicas(grp_system *s, int32_t n_replicas, uint6
     // at least 65,536 entries (every pair, for systems of up to ~360 atoms, whose density may still
     // change a lot: ions condensing in a periodic box), + the padding of the warps' partly filled chunks
     // (16 warps of a 512-thread block, 256 entries each)
-    r->nbl_cap = (int)(std::min(all, std::max(2 * cnt + 1024, (size_t)65536)) + 16 * 256);
+    // (a multiple of four words: every replica's list starts on 16 bytes)
+    r->nbl_cap = (int)((std::min(all, std::max(2 * cnt + 1024, (size_t)65536)) + 16 * 256 + 3) & ~(size_t)3);
     AL(r->nbl, R * (size_t)r->nbl_cap * 4);
     AL(r->qref, R * (size_t)n * 16);
     if (D.gb) {
@@ -1064,6 +1121,7 @@ static void fill_args(grp_batch *b, int k, const RunTick *ticks) {
     a.pairs_in_smem = r->sys->seg.pairs_in_smem;
     a.noise_batch = r->sys->seg.noise_batch;
     a.lean = r->sys->seg.lean;
+    a.charges_in_smem = r->sys->seg.charges_in_smem;
     b->h_args[i] = a;
   }
   for (int i = 0; i < nr; ++i) {

@@ -25,6 +25,11 @@ constexpr double kFixScale = 1099511627776.0;       // 2^40
 constexpr double kFixInv = 1.0 / 1099511627776.0;
 constexpr double kFixLimit = 4194304.0;               // 2^22
 
+// Mixed path: bonds at least this stiff (kJ/mol/nm^2) take r - r0 in double-single arithmetic.
+constexpr float kSoftBond = 1.0e4f;
+// Systems in vacuum on the mixed path keep neighbour rows from this size on.
+constexpr int kRowsMinAtoms = 1024;
+
 // Device copy of a system.  All arrays are device memory owned by grp_system.  Parameters exist in
 // FP64 (FP64 path) and FP32 (mixed path) copies.
 struct SysDev {
@@ -47,7 +52,19 @@ struct SysDev {
   int n_tiles, n_tile_pairs;
   const uint32_t *tile_pairs;  // I | J << 16
   const uint32_t *tile_masks;  // [n_tile_pairs][32]
+  // Neighbour rows (rows.cuh): for tiles I and J and atom i = 32 I + lane, the atoms of J on i's row: not excluded, and
+  // of i < j with i + j odd or i > j with i + j even
+  int use_rows;
+  const uint32_t *row_masks;   // [n_tiles][n_tiles][32]
+  // soft springs as static rows: partners, 0xFFFF for none; strengths and lengths of the same places; the remaining
+  // bonds by index
+  const int *spring_rows;      // [n_tiles] rows of a tile's longest atom
+  const ushort4 *spring_j;     // [rows / 4][n]
+  const float4 *spring_f;      // [rows / 4][n][2] (k, r0, k, r0)
+  int n_stiff;
+  const int *stiff;
   double cutoff2;          // 0: no cutoff
+  float cutoff2_f;
   int coulomb_rf;          // Coulomb model: 0 dielectric eps = 4r, 1 reaction field (eps_r = 1),
                            // 2 periodic: Ewald real space on pairs plus particle mesh Ewald
   int gb;                  // 1: Generalized Born (OBC II) implicit solvent
@@ -229,6 +246,17 @@ __device__ __forceinline__ Split to_split(float v, int *err) {
   *err |= (fabsf(v) < kSplitLimit) ? 0 : kErrOverflow;
   return s;
 }
+// The same split for |v| < 2^10 without conversions: a + 1.5 2^23 rounded down leaves floor(a) in the sum's
+// significand (|a| < 2^22), and r 2^20 + 2^23 rounded to nearest the rounded low word in its low bits (r 2^20 is
+// exact and at most 2^20).
+__device__ __forceinline__ Split to_split_small(float v) {
+  const float a = v * kSplitHiScale, t = __fadd_rd(a, 12582912.0f), r = a - __fsub_rn(t, 12582912.0f);
+  Split s;
+  s.hi = __float_as_int(t) - 0x4B400000;
+  s.lo = (unsigned int)__float_as_int(__fmaf_rn(r, kSplitLoScale, 8388608.0f)) - 0x4B000000u;
+  return s;
+}
+constexpr float kSplitSmall = 1024.0f;
 __device__ __forceinline__ long long split_value(Split s) { return (long long)s.hi * (1ll << 20) + (long long)s.lo; }
 __device__ __forceinline__ void split_add(int *hi, unsigned int *lo, int idx, Split s) {
   atomicAdd(&hi[idx], s.hi);

@@ -119,6 +119,7 @@ struct Params<PathF64> {
 template <>
 struct Params<PathMixed> {
   const float4 *atom;
+  const float *qc;      // the charges (third words of the table) side by side in shared memory; null: none
   const float2 *bond, *angle;
   const float4 *term;
   int rf;
@@ -384,9 +385,6 @@ __device__ __forceinline__ float bond_dr_ds(const Pos<PathMixed> &pos, int i, in
   return __fadd_rn(__fsub_rn(r, r0), rlo);
 }
 
-// Mixed path: bonds at least this stiff (kJ/mol/nm^2) take r - r0 in double-single arithmetic.
-constexpr float kSoftBond = 1.0e4f;
-
 // Harmonic bond 1/2 k (r - r0)^2: force on atom i (minus the force on j) and the energy.
 template <class P>
 __device__ __forceinline__ V3<typename P::T> bond_eval(const Pos<P> &pos, const Params<P> &par, int b, int i, int j,
@@ -553,6 +551,20 @@ __device__ __forceinline__ void list_pass(const SysDev &S, const Pos<P> &pos, co
   }
 }
 
+// Angles and dihedrals without the item table.
+template <class P>
+__device__ __forceinline__ void angle_dihedral_pass(const SysDev &S, const Pos<P> &pos, const Params<P> &par,
+                                                    const typename P::Acc &acc, bool want_e, long long &e_fix,
+                                                    int *err) {
+  const int bd = blockDim.x;
+  for (int t = threadIdx.x; t < S.n_angles; t += bd) {
+    const int4 ijk = S.angle_ijk[t];
+    angle_term<P>(pos, par, t, ijk.x, ijk.y, ijk.z, acc, want_e, e_fix, err);
+  }
+  for (int t = threadIdx.x; t < S.n_dih; t += bd)
+    dihedral_term<P>(pos, par, S.dih_ijkl[t], S.dih_terms[t], acc, want_e, e_fix, err);
+}
+
 // Bonded terms by kind, without the item table (large systems, whose tables stay in global memory):
 // each thread loads the indices and parameters of its next two bonds before evaluating them.
 template <class P>
@@ -566,12 +578,7 @@ __device__ __forceinline__ void bonded_pass(const SysDev &S, const Pos<P> &pos, 
     bond_term<P>(pos, par, b, ij0.x, ij0.y, acc, want_e, e_fix, err);
     if (b2 < S.n_bonds) bond_term<P>(pos, par, b2, ij1.x, ij1.y, acc, want_e, e_fix, err);
   }
-  for (int t = threadIdx.x; t < S.n_angles; t += bd) {
-    const int4 ijk = S.angle_ijk[t];
-    angle_term<P>(pos, par, t, ijk.x, ijk.y, ijk.z, acc, want_e, e_fix, err);
-  }
-  for (int t = threadIdx.x; t < S.n_dih; t += bd)
-    dihedral_term<P>(pos, par, S.dih_ijkl[t], S.dih_terms[t], acc, want_e, e_fix, err);
+  angle_dihedral_pass<P>(S, pos, par, acc, want_e, e_fix, err);
 }
 
 // One pass over every force-field item of a replica, strided over the block's threads.  The item

@@ -28,6 +28,7 @@ struct SegArgs {
   int pairs_in_smem;
   int noise_batch;           // steps of noise generated together (0: drawn inline per atom)
   int lean;                  // atom parameters read from the global table (large systems)
+  int charges_in_smem;       // the charges in an array of their own (neighbour rows)
   uint32_t *nbl;             // [R][nbl_cap] Verlet lists (systems with use_list), else null
   float4 *qref;              // [R][n] positions at the last list build
   int nbl_cap;
@@ -46,6 +47,7 @@ struct SegConfig {
   int pairs_in_smem;
   int noise_batch;
   int lean;
+  int charges_in_smem;
   // smaller blocks for many replicas (item-table systems): choice[0] = threads, and how many blocks of each size
   // the device holds at once
   int n_choices;

@@ -10,6 +10,7 @@
 #include "constraints.cuh"
 #include "gb.cuh"
 #include "pme.cuh"
+#include "rows.cuh"
 #include "kernels.h"
 #include "state.cuh"
 
@@ -294,6 +295,22 @@ __device__ int build_list(const SysDev &S, const State<P> &st, float *boxes, uin
   return c;
 }
 
+// The Verlet list of one replica in rows (or in pairs, when a row or the blocks had no room).
+__device__ __forceinline__ void build_row_list(const SysDev &S, const State<PathMixed> &st, float *boxes, uint32_t *pool,
+                                               int cap, RowList &L, float4 *qref, int *bins, int *cnt, int *err) {
+  tile_boxes<PathMixed>(S, st, boxes);
+  for (int at = threadIdx.x; at < S.n; at += blockDim.x) {
+    float x[3];
+    st.get_f32(at, x);
+    qref[at] = make_float4(x[0], x[1], x[2], 0.f);
+  }
+  L.n_pairs = -1;
+  if (!build_rows(S, st, boxes, pool, cap, L, bins, cnt)) {
+    L.n_pairs = build_list<PathMixed>(S, st, boxes, pool, cap, qref, cnt, err);
+    __syncthreads();
+  }
+}
+
 // Fixed-point sum (2^-40 units on the FP64 path, 2^-32 on the mixed path) to the path's precision,
 // the mixed path with 32-bit conversions only.
 __device__ __forceinline__ double fix_value(long long x, double) { return (double)x * kFixInv; }
@@ -367,7 +384,8 @@ enum : int {
   kModeAny = -1,   // decided per launch (the batched kernel, whose runs may differ)
   kModeItems = 0,  // explicit item table (fewer than 64 atoms)
   kModeTiles = 1,  // 32x32 atom tiles, no cutoff
-  kModeList = 2    // Verlet lists built from the tiles (cutoff)
+  kModeList = 2,   // Verlet lists built from the tiles (cutoff)
+  kModeRows = 3    // the same as neighbour rows (large systems, mixed path: S.use_rows)
 };
 
 // kFF: the nonbonded model compiled into the step loop, 0 = Coulomb with eps = 4r, 1 = reaction field,
@@ -399,9 +417,17 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
   // kFF = 5 (Verlet lists only): solvent and bond constraints together, the paper's protein-ligand setup
   constexpr bool kGB = kMode == kModeItems && kFF == 2;
   constexpr bool kGBL = kMode == kModeList && (kFF == 2 || kFF == 5);  // solvent with a cutoff on the list
-  constexpr bool kCon = (kMode == kModeItems && kFF == 3) || (kMode == kModeList && (kFF == 3 || kFF == 5));
+  constexpr bool kRows = kMode == kModeRows;
+  constexpr bool kCon = (kMode == kModeItems && kFF == 3) || (kMode == kModeList && (kFF == 3 || kFF == 5)) || (kRows && kFF == 3);
   constexpr bool kPME = (kMode == kModeItems || kMode == kModeList) && kFF == 4;
   constexpr int kRF = kFF == 4 ? 2 : (kFF >= 2 ? 0 : kFF);
+  float *qcs = nullptr;  // the charges side by side (rows)
+  if constexpr (kRows)
+    if (a.charges_in_smem) {
+      qcs = (float *)ptr;
+      ptr += (size_t)n * 4;
+      for (int i = threadIdx.x; i < n; i += kThreads) qcs[i] = S.atom_f[i].z;
+    }
   GbScratch<P> gbs;  // implicit solvent (item-table systems only)
   if constexpr (kGB) {
     ptr = align32(ptr);
@@ -450,18 +476,29 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
   __syncthreads();
   ObsAcc<P> oacc;
   if (threadIdx.x < no) oacc.begin(acc + 4 * threadIdx.x);
-  const bool use_list = kMode == kModeList || (kMode == kModeAny && a.nbl != nullptr);
-  const bool tiled = kMode == kModeTiles || kMode == kModeList || (kMode == kModeAny && S.tiled);
+  const bool use_list = kMode == kModeList || kRows || (kMode == kModeAny && a.nbl != nullptr);
+  const bool tiled = kMode == kModeTiles || kMode == kModeList || kRows || (kMode == kModeAny && S.tiled);
   const bool lean = kMode != kModeItems && a.lean;
   uint32_t *list = use_list ? a.nbl + (size_t)r * a.nbl_cap : nullptr;
   float4 *qref = use_list ? a.qref + (size_t)r * n : nullptr;
   int n_list = 0;
 
   int err = 0;
-  if (use_list) n_list = build_list<P>(S, st, boxes, list, a.nbl_cap, qref, lcount, &err);
+  RowList rl{list, n, 0, 0, 0, -1};
+  auto rebuild = [&](int *e) {
+    if constexpr (kRows) build_row_list(S, st, boxes, list, a.nbl_cap, rl, qref, reinterpret_cast<int *>(red), lcount, e);
+    else n_list = build_list<P>(S, st, boxes, list, a.nbl_cap, qref, lcount, e);
+  };
+  if constexpr (kRows) {
+    const RowPool rp = row_pool(S, a.nbl_cap);
+    rl.order = rp.order;
+    rl.chunks = rp.chunks;
+  }
+  if (use_list) rebuild(&err);
   const T h = (T)a.h, c1 = (T)a.c1;
   const Pos<P> pos = st.pos();
-  const Params<P> par = st.params(S);
+  Params<P> par = st.params(S);
+  if constexpr (kRows) par.qc = qcs;
   const typename P::Acc fa = State<P>::acc(F, n);
   // steps until the next sample: (t_phase0 + s + 1) % t_gr == 0
   int until = a.t_gr > 0 ? (int)(a.t_gr - a.t_phase0 % a.t_gr) : 0x7fffffff;
@@ -520,7 +557,7 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
       }
     }
     if (use_list) {
-      if (__syncthreads_or(moved)) n_list = build_list<P>(S, st, boxes, list, a.nbl_cap, qref, lcount, &err);
+      if (__syncthreads_or(moved)) rebuild(&err);
     } else {
       __syncthreads();
     }
@@ -558,6 +595,13 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
     if constexpr (kPME) pme_forces<P>(S, pos, par, fa, pms, sample, e_fix, &err);
     auto passes = [&](auto rf) {
       constexpr int R = decltype(rf)::value;
+      if constexpr (kRows) {
+        spring_rows(S, pos, par, fa, sample, e_fix, &err);
+        angle_dihedral_pass<P>(S, pos, par, fa, sample, e_fix, &err);
+        if (sample) visit_rows(rl, ListRow<R, true>(S, pos, par, fa, e_fix, &err));
+        else visit_rows(rl, ListRow<R, false>(S, pos, par, fa, e_fix, &err));
+        return;
+      }
       if (lean) bonded_pass<P>(S, pos, par, fa, sample, e_fix, &err);
       else force_pass<P, R>(S, pos, par, items, pairs, fa, sample, e_fix, &err);
       if (use_list) list_pass<P, R>(S, pos, par, list, n_list, fa, sample, e_fix, &err);
@@ -784,13 +828,14 @@ cudaError_t launch_noise_sd(const SysDev &S, double c1, double *sd_d, float *sd_
 }
 
 // ------------------------------------------------------------------------------------------------
-static size_t ff_smem_bytes(const SysDev &S, int pairs_in_smem, int noise_batch, int lean) {
+static size_t ff_smem_bytes(const SysDev &S, int pairs_in_smem, int noise_batch, int lean, int charges = 0) {
   const int n = S.n;
   const size_t real = S.precision == GRP_FP64 ? 8 : 4;
   size_t b = (size_t)3 * n * 8 + 64 * 8 + kMaxObs * 4 * 8 + 16 + 8 + 96;  // + alignment padding
   b += S.precision == GRP_FP64 ? State<PathF64>::bytes(n, lean) : State<PathMixed>::bytes(n, lean);
   b += (size_t)noise_batch * 3 * n * real;
   if (S.tiled && S.cutoff2 > 0) b += (size_t)S.n_tiles * 6 * 4;
+  if (charges) b += (size_t)n * 4;
   if (pairs_in_smem) b += (size_t)(S.n_pairs + S.n_items) * 4 + 32;
   if (S.gb && S.use_list) b += 32 + ScalarAcc<PathF64>::bytes(n);  // one 8-byte accumulator per atom
   else if (S.gb) b += 32 + (S.precision == GRP_FP64 ? GbScratch<PathF64>::bytes(n) : GbScratch<PathMixed>::bytes(n));
@@ -808,6 +853,10 @@ static auto ff_kernel(const SysDev &S, int threads) {
   // tiles are taken only without a cutoff, so never with the reaction field; implicit solvent only on
   // the item table (and never with a cutoff)
   const bool rf = S.coulomb_rf == 1, gb = S.gb != 0, con = S.n_cons > 0, pme = S.coulomb_rf == 2;
+  if constexpr (P::kMixed)
+    if (S.use_rows)
+      return rf ? ff_segment_kernel<P, 512, 1, kModeRows, 1>
+                : (con ? ff_segment_kernel<P, 512, 1, kModeRows, 3> : ff_segment_kernel<P, 512, 1, kModeRows, 0>);
   return mode == kModeItems
                   ? (pme  ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 4> : ff_segment_kernel<P, 512, 1, kModeItems, 4>)
                      : con ? (small ? ff_segment_kernel<P, 320, 2, kModeItems, 3> : ff_segment_kernel<P, 512, 1, kModeItems, 3>)
@@ -905,7 +954,8 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
     c.noise_batch = nb = 0;
   }
   c.pairs_in_smem = ff_smem_bytes(S, 1, nb, c.lean) <= 160 * 1024 ? 1 : 0;
-  c.smem = ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean);
+  c.charges_in_smem = S.use_rows && ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean, 1) <= kMaxSmem;
+  c.smem = ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean, c.charges_in_smem);
   c.n_choices = 1;
   c.choice[0] = c.threads;
   if (!S.tiled && S.coulomb_rf != 2 && threads_hint <= 0 && c.smem <= kMaxSmem) {
@@ -966,6 +1016,7 @@ cudaError_t launch_segment(const SegArgs &a0, const SegConfig &c, cudaStream_t s
   a.pairs_in_smem = c.pairs_in_smem;
   a.noise_batch = c.noise_batch;
   a.lean = c.lean;
+  a.charges_in_smem = c.charges_in_smem;
   if (a.n_active <= 0) return cudaSuccess;
   if (a.S.potential == GRP_POT_DOUBLE_WELL_2D) {
     return launch_dw(a, st);

@@ -172,7 +172,7 @@ struct State<PathMixed> {
   }
   __device__ Pos<PathMixed> pos() const { return Pos<PathMixed>{qh, ql}; }
   __device__ Params<PathMixed> params(const SysDev &S) const {
-    return Params<PathMixed>{atom, S.bond_f, S.angle_f, S.term_f, S.coulomb_rf, (float)S.krf, (float)S.crf,
+    return Params<PathMixed>{atom, nullptr, S.bond_f, S.angle_f, S.term_f, S.coulomb_rf, (float)S.krf, (float)S.crf,
                              {(float)S.box[0], (float)S.box[1], (float)S.box[2]},
                              {(float)S.ibox[0], (float)S.ibox[1], (float)S.ibox[2]}, (float)S.ewald_beta};
   }

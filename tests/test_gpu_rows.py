@@ -1,0 +1,84 @@
+"""Neighbour rows (large systems in vacuum on the mixed path) against the pair list of the batched kernel, which
+keeps it: the sums are integers, so the two agree bit for bit, over sizes around the tiles and the line between the
+two forms, with and without constraints and reaction field, through several rebuilds; and rows that outgrow their
+pieces (a dense clump) fall back to pairs."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_1807_02431_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+SEED = 2431
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_1807_02431_gb300 import binding
+
+    binding.load()
+    return binding
+
+
+def _pair(B, s, R, k, t_gr, seed=6):
+    """The same replicas advanced alone (rows) and in a batch of one run (pairs)."""
+    q0, p0 = W.replica_states(s, R, seed=seed, spread=0.002)
+    sysh = B.grp_create_system(s, B.GRP_MIXED)
+    alone, run = (B.grp_init_replicas(sysh, R, SEED, q0, p0, per_replica=True) for _ in range(2))
+    B.grp_step_k(alone, k, t_gr)
+    B.grp_batch_step_k(B.grp_batch_create([run]), k, t_gr)
+    return B.grp_get_state(alone)[:3], B.grp_get_state(run)[:3]
+
+
+@pytest.mark.parametrize("n,rf", [(993, False), (994, False), (995, True), (1023, False), (1500, True), (1840, False),
+                                  (2000, False), (2100, True)])
+def test_rows_give_the_bits_of_the_pair_list(B, n, rf):
+    s = W.ligand_receptor(n_receptor=n)
+    if rf:
+        s = dataclasses.replace(s, coulomb_mode=W.COULOMB_REACTION_FIELD)
+    for a, b in zip(*_pair(B, s, 3, 120, 20)):
+        assert np.array_equal(a, b)
+
+
+def test_rows_with_constraints(B, oracle_mod):
+    """Constrained hydrogens are not batched: one step against the FP64 oracle, with the tolerances of the other
+    one-step tests of the mixed path."""
+    s = W.ligand_receptor_h()
+    q0, p0 = W.replica_states(s, 2, seed=4, spread=0.0)
+    rep = B.grp_init_replicas(B.grp_create_system(s, B.GRP_MIXED), 2, SEED, q0, p0, per_replica=True)
+    B.grp_step_k(rep, 1, 0)
+    q, p = B.grp_get_state(rep)[:2]
+    o = oracle_mod.Oracle(s)
+    qo, po = q0.copy(), p0.copy()
+    fo = np.stack([o.forces(qo[r]) for r in range(2)])
+    o.step_k(qo, po, fo, SEED, 0, 0, 1, 0, cap=1)
+    assert np.abs(q - qo).max() <= 1e-9 * np.abs(qo).max() and np.abs(p - po).max() <= 1e-6 * np.abs(po).max()
+
+
+@pytest.fixture(scope="module")
+def oracle_mod():
+    import oracle
+
+    oracle.build()
+    return oracle
+
+
+@pytest.mark.parametrize("side", [0, 8, 10])
+def test_dense_clumps(B, side):
+    """A clump of side^3 weakly charged beads on a lattice of 0.12 nm (no Lennard-Jones) in a sparse gas: up to 1,000
+    partners within the cutoff, more than a row's 256 places or the pool's blocks, beside a sparse rest.  The largest
+    force is some ten kJ/mol/nm."""
+    n = 1100
+    rng = np.random.default_rng(3)
+    x = np.stack(np.meshgrid(*[np.arange(11)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n] * 0.9
+    m = side ** 3
+    if m:
+        x[:m] = 20.0 + 0.12 * np.stack(np.meshgrid(*[np.arange(side)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    s = W.System(name="gas", n_atoms=n, dim=3, potential=W.POT_FORCE_FIELD, mass=np.full(n, 12.0), kT=0.1, gamma=1.0,
+                 dt=0.002, sigma=np.full(n, 0.05), epsilon=np.zeros(n), charge=rng.normal(0, 0.01, n),
+                 excl=np.zeros((0, 2), np.int32), cutoff=1.2, coulomb_k=W.COULOMB_K, cv_kind=W.CV_COM_DISTANCE,
+                 cv_params=(1.0,), groups=[[0], [1]], observables=[(W.OBS_POTENTIAL, ()), (W.OBS_KINETIC, ())])
+    s.q0, s.p0 = x, W.maxwell_boltzmann(s.mass, s.kT, 3, rng)
+    for a, b in zip(*_pair(B, s, 2, 40, 10)):
+        assert np.array_equal(a, b)
