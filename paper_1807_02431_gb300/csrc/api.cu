@@ -752,6 +752,13 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
     s->theta = const_cast<double *>(dth);
   }
 #undef UP
+  D.f32.krf = (float)D.krf;
+  D.f32.crf = (float)D.crf;
+  for (int x = 0; x < 3; ++x) {
+    D.f32.box[x] = (float)D.box[x];
+    D.f32.ibox[x] = (float)D.ibox[x];
+  }
+  D.f32.ewald_beta = (float)D.ewald_beta;
   s->seg = segment_config(D, 0);
   if (s->seg.smem > kMaxSmem) {
     grp_destroy_system(s);

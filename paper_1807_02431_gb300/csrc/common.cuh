@@ -30,10 +30,19 @@ constexpr float kSoftBond = 1.0e4f;
 // Systems in vacuum on the mixed path keep neighbour rows from this size on.
 constexpr int kRowsMinAtoms = 1024;
 
+// Scalars of a system rounded to FP32 on the host, for the pair loops of the mixed path: a conversion in the kernel
+// is an instruction at the FP64 pipe's rate, and under register pressure the compiler repeats it where the value is
+// used.  With gnearest (forcefield.cuh): 220 atoms in a periodic box, 256 replicas x 500 steps, 25.6 -> 24.8 ms.
+struct SysF32 {
+  float krf, crf;
+  float box[3], ibox[3], ewald_beta;
+};
+
 // Device copy of a system.  All arrays are device memory owned by grp_system.  Parameters exist in
 // FP64 (FP64 path) and FP32 (mixed path) copies.
 struct SysDev {
   int n, dim, nd, potential, precision;
+  SysF32 f32;
   double dw_a, dw_b;
   double kT, gamma, dt;
   const double *mass;      // [n]

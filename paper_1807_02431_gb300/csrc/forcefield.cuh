@@ -153,7 +153,9 @@ __device__ __forceinline__ float gerfc_e(float x, float e) {
 __device__ __forceinline__ double gerf(double x) { return erf(x); }
 __device__ __forceinline__ float gerf(float x) { return erff(x); }
 __device__ __forceinline__ double gnearest(double x) { return rint(x); }
-__device__ __forceinline__ float gnearest(float x) { return rintf(x); }
+// (|x| < 2^22: adding 1.5 2^23 leaves the nearest integer, ties to even, in the sum's significand; the rounding
+// instruction shares the FP64 pipe's rate.  Differences of more boxes have no digits of a box left in FP32.)
+__device__ __forceinline__ float gnearest(float x) { return __fsub_rn(__fadd_rn(x, 12582912.0f), 12582912.0f); }
 
 template <int kRF, class T, class Par>
 __device__ __forceinline__ T pair_g(const Par &par, T eps, T s6, T qq, T r2, T inv_r2) {

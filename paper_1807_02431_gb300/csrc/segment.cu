@@ -226,8 +226,8 @@ __device__ int build_list(const SysDev &S, const State<P> &st, float *boxes, uin
   // periodic box: tile gaps and pair distances over nearest images (cutoff + skin is at most half the
   // shortest edge, so a pair within it has one nearest image)
   const bool per = S.coulomb_rf == 2;
-  const float L[3] = {(float)S.box[0], (float)S.box[1], (float)S.box[2]};
-  const float iL[3] = {(float)S.ibox[0], (float)S.ibox[1], (float)S.ibox[2]};
+  const float L[3] = {S.f32.box[0], S.f32.box[1], S.f32.box[2]};
+  const float iL[3] = {S.f32.ibox[0], S.f32.ibox[1], S.f32.ibox[2]};
   int wpos = 0, wleft = 0;  // this warp's next free entry and the room left in its chunk (warp-uniform)
   for (int tp = warp; tp < S.n_tile_pairs; tp += nwarps) {
     const uint32_t e = S.tile_pairs[tp];

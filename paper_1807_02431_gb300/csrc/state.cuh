@@ -172,9 +172,9 @@ struct State<PathMixed> {
   }
   __device__ Pos<PathMixed> pos() const { return Pos<PathMixed>{qh, ql}; }
   __device__ Params<PathMixed> params(const SysDev &S) const {
-    return Params<PathMixed>{atom, nullptr, S.bond_f, S.angle_f, S.term_f, S.coulomb_rf, (float)S.krf, (float)S.crf,
-                             {(float)S.box[0], (float)S.box[1], (float)S.box[2]},
-                             {(float)S.ibox[0], (float)S.ibox[1], (float)S.ibox[2]}, (float)S.ewald_beta};
+    return Params<PathMixed>{atom, nullptr, S.bond_f, S.angle_f, S.term_f, S.coulomb_rf, S.f32.krf, S.f32.crf,
+                             {S.f32.box[0], S.f32.box[1], S.f32.box[2]},
+                             {S.f32.ibox[0], S.f32.ibox[1], S.f32.ibox[2]}, S.f32.ewald_beta};
   }
   __device__ __forceinline__ void baoa(int at, const float *xi, float h, float c1) {
     const float im = atom[at].w, s = sd[at], hm = h * im;
