@@ -77,25 +77,46 @@ __device__ __forceinline__ auto gb_atom(const SysDev &S, int i) {
 // The solvent forces (and energy when want_e) of one replica, added to the force accumulators; called
 // by every thread of the block, with the positions final; returns after the last pass (the caller's
 // barrier before reading the forces covers it).  The scratch accumulators are zero on entry and left
-// zero.
-template <class P>
-__device__ void gb_forces(const SysDev &S, const Pos<P> &pos, const typename P::Acc &fa, const GbScratch<P> &g,
-                          bool want_e, long long &e_fix, int *err) {
+// zero.  A step of such a small system is a chain of latencies, so
+//  * each thread's first pair (the only one up to 25 beads on 320 threads) keeps its difference, distance, charges and
+//    derivatives in registers through the three pair passes;
+//  * `other()`, the vacuum forces, runs beside pass 2, whose one warp of atoms with divisions and a hyperbolic
+//    tangent would keep the rest of the block waiting.
+// 22 beads, 256 replicas x 500 steps: 2.10 -> 1.94 ms.
+template <class P, class Other>
+__device__ __forceinline__ void gb_forces(const SysDev &S, const Pos<P> &pos, const typename P::Acc &fa, const GbScratch<P> &g,
+                          bool want_e, long long &e_fix, int *err, Other other) {
   using T = typename P::T;
   const int n = S.n, np = S.n_gb_pairs, bd = blockDim.x;
   const T tau = (T)S.gb_tau;
-  // 1. descreening sums
-  for (int t = threadIdx.x; t < np; t += bd) {
+  struct Pair {
+    int i, j;
+    V3<T> d;
+    T r2, r, qq, dhij, dhji;
+  };
+  auto load = [&](int t, Pair &p) {
     const uint32_t pk = S.gb_pairs[t];
-    const int i = (int)(pk & 0xFFFFu), j = (int)(pk >> 16);
-    const V3<T> d = pos.diff(i, j);
-    const T r = gsqrt(dot(d, d));
-    const auto pi = gb_atom<P>(S, i), pj = gb_atom<P>(S, j);
-    T dhij, dhji;
-    g.acc.add(i, gb_hct<T>(r, (T)pi.x, (T)pj.z, dhij), err);
-    g.acc.add(j, gb_hct<T>(r, (T)pj.x, (T)pi.z, dhji), err);
-    g.dh[2 * t] = dhij;  // kept for the chain rule (pass 5)
-    g.dh[2 * t + 1] = dhji;
+    p.i = (int)(pk & 0xFFFFu);
+    p.j = (int)(pk >> 16);
+    p.d = pos.diff(p.i, p.j);
+    p.r2 = dot(p.d, p.d);
+    p.r = gsqrt(p.r2);
+  };
+  Pair first;
+  // 1. descreening sums
+  auto descreen = [&](int t, Pair &p) {
+    load(t, p);
+    const auto pi = gb_atom<P>(S, p.i), pj = gb_atom<P>(S, p.j);
+    p.qq = (T)pi.w * (T)pj.w;
+    g.acc.add(p.i, gb_hct<T>(p.r, (T)pi.x, (T)pj.z, p.dhij), err);
+    g.acc.add(p.j, gb_hct<T>(p.r, (T)pj.x, (T)pi.z, p.dhji), err);
+  };
+  if (threadIdx.x < np) descreen(threadIdx.x, first);
+  for (int t = threadIdx.x + bd; t < np; t += bd) {
+    Pair p;
+    descreen(t, p);
+    g.dh[2 * t] = p.dhij;  // kept for the chain rule (pass 5)
+    g.dh[2 * t + 1] = p.dhji;
   }
   __syncthreads();
   // 2. Born radii, dB/dI, the self terms of E and dE/dB
@@ -111,23 +132,27 @@ __device__ void gb_forces(const SysDev &S, const Pos<P> &pos, const typename P::
     g.acc.set(n + i, T(0.5) * tau * qi * qi / (B * B), err);
     if (want_e) e_fix += fa.efix(T(-0.5) * tau * qi * qi / B, err);
   }
+  other();
   __syncthreads();
   // 3. pair terms at fixed Born radii: forces and the pairs' parts of dE/dB
-  for (int t = threadIdx.x; t < np; t += bd) {
-    const uint32_t pk = S.gb_pairs[t];
-    const int i = (int)(pk & 0xFFFFu), j = (int)(pk >> 16);
-    const V3<T> d = pos.diff(i, j);
-    const T r2 = dot(d, d);
-    const T bi = g.born[i], bj = g.born[j], bb = bi * bj, D = r2 / (T(4) * bb), e = gexp(-D);
-    const T f2 = r2 + bb * e, f = gsqrt(f2), qq = (T)gb_atom<P>(S, i).w * (T)gb_atom<P>(S, j).w;
-    const T dEdf = tau * qq / f2;
+  auto pair_terms = [&](const Pair &p) {
+    const T bi = g.born[p.i], bj = g.born[p.j], bb = bi * bj, D = p.r2 / (T(4) * bb), e = gexp(-D);
+    const T f2 = p.r2 + bb * e, f = gsqrt(f2);
+    const T dEdf = tau * p.qq / f2;
     const T dBcommon = dEdf * e * (T(1) + D) / (T(2) * f);
-    g.acc.add(n + i, dBcommon * bj, err);
-    g.acc.add(n + j, dBcommon * bi, err);
+    g.acc.add(n + p.i, dBcommon * bj, err);
+    g.acc.add(n + p.j, dBcommon * bi, err);
     const T gr = -dEdf * (T(1) - T(0.25) * e) / f;  // -dE/dr / r
-    fa.add(i, V3<T>{gr * d.x, gr * d.y, gr * d.z}, err);
-    fa.add(j, V3<T>{-gr * d.x, -gr * d.y, -gr * d.z}, err);
-    if (want_e) e_fix += fa.efix(-tau * qq / f, err);
+    fa.add(p.i, V3<T>{gr * p.d.x, gr * p.d.y, gr * p.d.z}, err);
+    fa.add(p.j, V3<T>{-gr * p.d.x, -gr * p.d.y, -gr * p.d.z}, err);
+    if (want_e) e_fix += fa.efix(-tau * p.qq / f, err);
+  };
+  if (threadIdx.x < np) pair_terms(first);
+  for (int t = threadIdx.x + bd; t < np; t += bd) {
+    Pair p;
+    load(t, p);
+    p.qq = (T)gb_atom<P>(S, p.i).w * (T)gb_atom<P>(S, p.j).w;
+    pair_terms(p);
   }
   __syncthreads();
   // 4. chain-rule weights w_i = dE/dB_i dB_i/dI_i / 2
@@ -137,14 +162,18 @@ __device__ void gb_forces(const SysDev &S, const Pos<P> &pos, const typename P::
   }
   __syncthreads();
   // 5. forces through the Born radii
-  for (int t = threadIdx.x; t < np; t += bd) {
-    const uint32_t pk = S.gb_pairs[t];
-    const int i = (int)(pk & 0xFFFFu), j = (int)(pk >> 16);
-    const V3<T> d = pos.diff(i, j);
-    const T r = gsqrt(dot(d, d));
-    const T gr = -(g.w[i] * g.dh[2 * t] + g.w[j] * g.dh[2 * t + 1]) / r;
-    fa.add(i, V3<T>{gr * d.x, gr * d.y, gr * d.z}, err);
-    fa.add(j, V3<T>{-gr * d.x, -gr * d.y, -gr * d.z}, err);
+  auto chain_rule = [&](const Pair &p) {
+    const T gr = -(g.w[p.i] * p.dhij + g.w[p.j] * p.dhji) / p.r;
+    fa.add(p.i, V3<T>{gr * p.d.x, gr * p.d.y, gr * p.d.z}, err);
+    fa.add(p.j, V3<T>{-gr * p.d.x, -gr * p.d.y, -gr * p.d.z}, err);
+  };
+  if (threadIdx.x < np) chain_rule(first);
+  for (int t = threadIdx.x + bd; t < np; t += bd) {
+    Pair p;
+    load(t, p);
+    p.dhij = g.dh[2 * t];
+    p.dhji = g.dh[2 * t + 1];
+    chain_rule(p);
   }
 }
 

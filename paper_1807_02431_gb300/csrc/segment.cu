@@ -568,7 +568,9 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
     const bool sample = --until == 0;
     if (sample) until = a.t_gr;
     long long e_fix = 0;
-    if constexpr (kGB) gb_forces<P>(S, pos, fa, gbs, sample, e_fix, &err);
+    if constexpr (kGB)  // the vacuum forces (items) run beside the Born radii
+      gb_forces<P>(S, pos, fa, gbs, sample, e_fix, &err,
+                   [&]() { force_pass<P, kRF>(S, pos, par, items, pairs, fa, sample, e_fix, &err); });
     if constexpr (kGBL) {
       const int nl = n_list;
       // batches of kGbBatch entries per thread (list entries t, t + kThreads, ...), padding entries and
@@ -607,7 +609,8 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
       if (use_list) list_pass<P, R>(S, pos, par, list, n_list, fa, sample, e_fix, &err);
       else if (tiled) tile_pass<P, false, R>(S, pos, par, fa, boxes, sample, e_fix, &err);  // tiles: no cutoff
     };
-    if constexpr (kRF >= 0) {
+    if constexpr (kGB) {
+    } else if constexpr (kRF >= 0) {
       passes(std::integral_constant<int, kRF>{});
     } else if (par.rf) {
       passes(std::integral_constant<int, 1>{});
@@ -1092,7 +1095,7 @@ __global__ void __launch_bounds__(256) energy_forces_kernel(SysDev S, const doub
     }, energy != nullptr, e_fix, &err);
     __syncthreads();
   } else if (S.gb) {
-    gb_forces<P>(S, st.pos(), fa, gbs, energy != nullptr, e_fix, &err);
+    gb_forces<P>(S, st.pos(), fa, gbs, energy != nullptr, e_fix, &err, []() {});
   }
   if (S.coulomb_rf == 2) pme_forces<P>(S, st.pos(), st.params(S), fa, pms, energy != nullptr, e_fix, &err);
   force_pass<P>(S, st.pos(), st.params(S), S.items, S.pairs, fa, energy != nullptr, e_fix, &err);
