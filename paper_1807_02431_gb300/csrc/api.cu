@@ -420,7 +420,7 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
       bd[b] = make_double2(d->bond_k[b], d->bond_r0[b]);
       bf[b] = make_float2((float)bd[b].x, (float)bd[b].y);
     }
-    // Large systems evaluate their bonds straight from these arrays, 32 consecutive bonds per warp: order
+    // Large systems (without neighbour rows) evaluate their bonds straight from these arrays, 32 consecutive bonds per warp: order
     // them in greedy rounds of atom-disjoint bonds, so that a warp's fixed-point additions go to distinct
     // atoms (the elastic network's springs come atom by atom, and consecutive springs of one atom made
     // the lanes of a warp add to the same words: 90,000 -> 63,000 cycles per step of the ligand's

@@ -553,6 +553,33 @@ __device__ __forceinline__ void list_pass(const SysDev &S, const Pos<P> &pos, co
   }
 }
 
+// The FP64 path's dihedrals as a function of its own: inlined, the compiler contracted its products and sums in one way
+// in the batched kernel and in another in the single-run kernels (1 ulp of a force), and a run in a batch has to be the
+// run alone bit for bit.  The call costs 3 % (22 beads, 256 replicas x 500 steps, 7.07 -> 7.29 ms).
+struct DihedralDone {
+  long long e;
+  int err;
+};
+static __device__ __noinline__ DihedralDone dihedral_f64(const double *q, const double4 *terms, int4 a, int2 range, long long *F,
+                                                         bool want_e) {
+  Params<PathF64> par{};
+  par.term = terms;
+  DihedralDone d{0, 0};
+  dihedral_term<PathF64>(Pos<PathF64>{q}, par, a, range, AccF64{F}, want_e, d.e, &d.err);
+  return d;
+}
+template <class P>
+__device__ __forceinline__ void dihedral_item(const Pos<P> &pos, const Params<P> &par, int4 a, int2 terms,
+                                              const typename P::Acc &acc, bool want_e, long long &e_fix, int *err) {
+  if constexpr (std::is_same<P, PathF64>::value) {
+    const DihedralDone d = dihedral_f64(pos.q, par.term, a, terms, acc.F, want_e);
+    e_fix += d.e;
+    *err |= d.err;
+  } else {
+    dihedral_term<P>(pos, par, a, terms, acc, want_e, e_fix, err);
+  }
+}
+
 // Angles and dihedrals without the item table.
 template <class P>
 __device__ __forceinline__ void angle_dihedral_pass(const SysDev &S, const Pos<P> &pos, const Params<P> &par,
@@ -564,7 +591,7 @@ __device__ __forceinline__ void angle_dihedral_pass(const SysDev &S, const Pos<P
     angle_term<P>(pos, par, t, ijk.x, ijk.y, ijk.z, acc, want_e, e_fix, err);
   }
   for (int t = threadIdx.x; t < S.n_dih; t += bd)
-    dihedral_term<P>(pos, par, S.dih_ijkl[t], S.dih_terms[t], acc, want_e, e_fix, err);
+    dihedral_item<P>(pos, par, S.dih_ijkl[t], S.dih_terms[t], acc, want_e, e_fix, err);
 }
 
 // Bonded terms by kind, without the item table (large systems, whose tables stay in global memory):
@@ -607,7 +634,7 @@ __device__ __forceinline__ void force_pass(const SysDev &S, const Pos<P> &pos, c
       const int4 ijk = S.angle_ijk[idx];
       angle_term<P>(pos, par, idx, ijk.x, ijk.y, ijk.z, acc, want_e, e_fix, err);
     } else if (kind == kItemDihedral) {
-      dihedral_term<P>(pos, par, S.dih_ijkl[idx], S.dih_terms[idx], acc, want_e, e_fix, err);
+      dihedral_item<P>(pos, par, S.dih_ijkl[idx], S.dih_terms[idx], acc, want_e, e_fix, err);
     }
   }
 }
