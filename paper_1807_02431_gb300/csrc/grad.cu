@@ -153,11 +153,54 @@ __device__ __forceinline__ void param_pass(const SysDev &S, const A *atom, const
   }
 }
 
+// The positions of one configuration as digits of one fixed point: with 2^E above every coordinate, x 2^(62-E) rounded to
+// an integer (every bit of an FP64 coordinate next to 2^E, and 2^-53 length units for the others while E <= 10) and cut
+// into hi, units of 2^(E-23), mid, 24 bits, both as FP32 numbers, and lo, 15 bits.  Differences of each digit are
+// exact, and their sum is the difference rounded to FP32, as an FP64 subtraction and a conversion give it (the
+// same FP32 number in 11.8 million random differences; double-single numbers, 48 bits, were off by up to 32 ulp of a
+// difference at an offset of 60, 1,536 at 1,023).  Layout: (hi.xyz, lo.x | lo.y << 16), (mid.xyz, lo.z).
+struct Digits {
+  float4 *h, *m;
+  float unit;  // 2^(E-62)
+  __device__ __forceinline__ void store(int i, const double *x, int E) const {
+    const float uh = scalbnf(1.0f, E - 23), um = scalbnf(1.0f, E - 47);
+    float a[3], b[3];
+    unsigned int c[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int w = __double2hiint(x[k]), mag = w & 0x7FFFFFFF;
+      const unsigned long long f = ((unsigned long long)((mag & 0xFFFFF) | 0x100000) << 32) | (unsigned int)__double2loint(x[k]);
+      const long long v = fix_shift(f, (mag >> 20) - 1013 - E, w < 0);
+      a[k] = (float)(int)(v >> 39) * uh;
+      b[k] = (float)((int)(v >> 15) & 0xFFFFFF) * um;
+      c[k] = (unsigned int)v & 0x7FFFu;
+    }
+    h[i] = make_float4(a[0], a[1], a[2], __uint_as_float(c[0] | (c[1] << 16)));
+    m[i] = make_float4(b[0], b[1], b[2], __uint_as_float(c[2]));
+  }
+  __device__ __forceinline__ V3<float> diff(int i, int j) const {
+    const float4 a = h[i], b = h[j], c = m[i], d = m[j];
+    const int al = __float_as_int(a.w), bl = __float_as_int(b.w);
+    // t + e is the sum of the first two digits' differences without error: mid's is less than one unit of hi's, so hi's
+    // is the larger one or zero
+    auto sub = [&](float ah, float bh, float am, float bm, int lo) {
+      const float s = __fsub_rn(ah, bh), r = __fsub_rn(am, bm), t = __fadd_rn(s, r), e = __fsub_rn(r, __fsub_rn(t, s));
+      const float l = __fsub_rn(__int_as_float(0x4B400000 + lo), 12582912.0f);  // (float)lo, |lo| < 2^22
+      return __fadd_rn(t, __fmaf_rn(l, unit, e));
+    };
+    return {sub(a.x, b.x, c.x, d.x, (al & 0xFFFF) - (bl & 0xFFFF)), sub(a.y, b.y, c.y, d.y, (al >> 16) - (bl >> 16)),
+            sub(a.z, b.z, c.z, d.z, __float_as_int(c.w) - __float_as_int(d.w))};
+  }
+};
+// The range of E that takes the digits.
+constexpr int kDigitsMin = -16, kDigitsMax = 10;
+
 // One block per configuration b; G[2n + n_terms] fixed-point accumulators in shared memory.
-// kStaged (mixed path, where it fits): the positions wait in shared memory as double-single numbers and their
-// differences are formed in FP32.  An FP64 subtraction and conversion per coordinate and pair cost six instructions of
+// kStaged (mixed path, where it fits): the positions wait in shared memory as the digits above and their differences
+// are formed in FP32.  An FP64 subtraction and conversion per coordinate and pair cost six instructions of
 // the FP64 pipe (1/64 of the FP32 rate) and three 8-byte loads per atom from memory: energies and gradients of
-// 2,048 configurations of 100 beads 396 -> 285 us.
+// 2,048 configurations of 100 beads 396 -> 273 us.  A configuration whose largest coordinate is outside the digits'
+// range (or not finite) takes FP64 differences.
 template <class T, class A, class A4T, bool kStaged>
 __global__ void __launch_bounds__(256) param_grad_kernel(const __grid_constant__ SysDev S, const A *atom, const A4T *term,
                                                          int n_terms, const double *q, const double *w, double *grad_q,
@@ -166,26 +209,29 @@ __global__ void __launch_bounds__(256) param_grad_kernel(const __grid_constant__
   const int n = S.n, nt = 2 * n + n_terms, b = blockIdx.x;
   const double *qb = q + (size_t)b * S.nd;
   for (int i = threadIdx.x; i < nt; i += blockDim.x) G[i] = 0;
-  float4 *hi = reinterpret_cast<float4 *>(G + ((nt + 1) & ~1)), *lo = hi + n;
-  if constexpr (kStaged)
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const ds x = ds_from_double(qb[3 * i]), y = ds_from_double(qb[3 * i + 1]), v = ds_from_double(qb[3 * i + 2]);
-      hi[i] = make_float4(x.hi, y.hi, v.hi, 0.f);
-      lo[i] = make_float4(x.lo, y.lo, v.lo, 0.f);
-    }
-  __syncthreads();
   int err = 0;
   if constexpr (kStaged) {
-    auto sub = [](float ah, float al, float bh, float bl) {
-      const float s = __fsub_rn(ah, bh), bp = __fsub_rn(s, ah);
-      const float e = __fadd_rn(__fsub_rn(ah, __fsub_rn(s, bp)), __fsub_rn(-bh, bp));  // TwoSum(a, -b)
-      return __fadd_rn(s, __fadd_rn(e, __fsub_rn(al, bl)));
-    };
-    param_pass<T>(S, atom, term, [&](int i, int j) {
-      const float4 a = hi[i], b = hi[j], c = lo[i], d = lo[j];
-      return V3<T>{sub(a.x, c.x, b.x, d.x), sub(a.y, c.y, b.y, d.y), sub(a.z, c.z, b.z, d.z)};
-    }, ParamAcc{G}, &err);
+    float4 *h = reinterpret_cast<float4 *>(G + ((nt + 1) & ~1));
+    int *top = reinterpret_cast<int *>(h);  // the largest coordinate's high word, before the digits are there
+    if (threadIdx.x == 0) *top = 0;
+    __syncthreads();
+    int t = 0;
+    for (int i = threadIdx.x; i < S.nd; i += blockDim.x) t = max(t, __double2hiint(qb[i]) & 0x7FFFFFFF);
+    t = __reduce_max_sync(0xffffffffu, t);
+    if ((threadIdx.x & 31) == 0) atomicMax(top, t);
+    __syncthreads();
+    const int E = (*top >> 20) - 1022;  // every |coordinate| < 2^E
+    __syncthreads();
+    if (E >= kDigitsMin && E <= kDigitsMax) {
+      const Digits dg{h, h + n, scalbnf(1.0f, E - 62)};
+      for (int i = threadIdx.x; i < n; i += blockDim.x) dg.store(i, qb + 3 * i, E);
+      __syncthreads();
+      param_pass<T>(S, atom, term, [&](int i, int j) { return dg.diff(i, j); }, ParamAcc{G}, &err);
+    } else {
+      param_pass<T>(S, atom, term, [&](int i, int j) { return qdiff<T>(qb, i, j); }, ParamAcc{G}, &err);
+    }
   } else {
+    __syncthreads();
     param_pass<T>(S, atom, term, [&](int i, int j) { return qdiff<T>(qb, i, j); }, ParamAcc{G}, &err);
   }
   __syncthreads();

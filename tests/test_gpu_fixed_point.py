@@ -89,3 +89,22 @@ def test_param_gradient_against_autograd(B, n):
     want = [v.numpy() for v in torch.autograd.grad(e.sum(), (sig, eps))]
     for w, g, m in zip(want, (got[:n].cpu().numpy(), got[n:2 * n].cpu().numpy()), size):
         assert np.abs(g - w).max() <= 1e-6 * m
+
+
+@pytest.mark.parametrize("n", [22, 70, 100])
+@pytest.mark.parametrize("shift,grid", [(2.0 ** 6, 2.0 ** -44), (-2.0 ** 9, 2.0 ** -42), (2.0 ** 10, 2.0 ** -41),
+                                        (2.0 ** 30, 2.0 ** -20)])
+def test_param_gradient_of_shifted_positions(B, n, shift, grid):
+    """The mixed path's parameter gradient takes differences of whole FP64 positions: configurations on a grid that
+    FP64 still resolves after the shift have the same differences there, and so the same gradient bit for bit (on both
+    sides of the range in which the positions are held as FP32 digits)."""
+    import torch
+
+    s = W.chain(n)
+    sysh = B.grp_create_system(s, B.GRP_MIXED)
+    q = np.rint(W.replica_states(s, 16, seed=8, spread=0.01)[0] / grid) * grid
+    assert np.array_equal((q + shift) - shift, q)
+    here, there = (torch.empty(B.grp_param_count(sysh), dtype=torch.float64, device="cuda") for _ in range(2))
+    B.grp_energy_grad(sysh, 16, torch.from_numpy(q).cuda(), None, None, None, here)
+    B.grp_energy_grad(sysh, 16, torch.from_numpy(q + shift).cuda(), None, None, None, there)
+    assert torch.equal(here, there)
