@@ -278,6 +278,7 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
   grp_system *s = new grp_system();
   CU(cudaGetDevice(&s->device));
   SysDev &D = s->dev;
+  RowsDev rows{};
   D.n = n;
   D.dim = d->dim;
   D.nd = n * d->dim;
@@ -340,7 +341,7 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
       excl[(size_t)i * n + j] = excl[(size_t)j * n + i] = 1;
     }
     D.cutoff2 = d->cutoff > 0 ? d->cutoff * d->cutoff : 0.0;
-    D.cutoff2_f = (float)D.cutoff2;
+    rows.cutoff2 = (float)D.cutoff2;
     if (d->coulomb_mode == GRP_COULOMB_REACTION_FIELD) {
       if (!(d->cutoff > 0)) { grp_destroy_system(s); return fail(GRP_EINVAL, "the reaction field needs cutoff > 0"); }
       if (!(d->rf_dielectric == 0.0 || d->rf_dielectric >= 1.0)) {
@@ -486,11 +487,11 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
       const StaticRows sr = static_rows(soft);
       std::vector<float2> kf(sr.partner.size(), make_float2(0.f, 0.f));
       for (size_t u = 0; u < soft.size(); ++u) kf[sr.place[u]] = bf[index[u]];
-      UP(sr.tile_rows.data(), sr.tile_rows.size(), &D.spring_rows);
-      UP(reinterpret_cast<const ushort4 *>(sr.partner.data()), sr.partner.size() / 4, &D.spring_j);
-      UP(reinterpret_cast<const float4 *>(kf.data()), kf.size() / 2, &D.spring_f);
-      D.n_stiff = (int)stiff.size();
-      UP(stiff.data(), stiff.size(), &D.stiff);
+      UP(sr.tile_rows.data(), sr.tile_rows.size(), &rows.spring_rows);
+      UP(reinterpret_cast<const ushort4 *>(sr.partner.data()), sr.partner.size() / 4, &rows.spring_j);
+      UP(reinterpret_cast<const float4 *>(kf.data()), kf.size() / 2, &rows.spring_f);
+      rows.n_stiff = (int)stiff.size();
+      UP(stiff.data(), stiff.size(), &rows.stiff);
       // a pair is on the row of its lower atom when the sum of the two is odd, of the higher when it is even, so
       // that every atom has about half of its neighbours on its row
       const int nt = D.n_tiles;
@@ -499,7 +500,7 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
         for (int j = 0; j < n; ++j)
           if (i != j && !excl[(size_t)i * n + j] && (((i + j) & 1) ? i < j : i > j))
             rmask[((size_t)(i / 32) * nt + j / 32) * 32 + i % 32] |= 1u << (j % 32);
-      UP(rmask.data(), rmask.size(), &D.row_masks);
+      UP(rmask.data(), rmask.size(), &rows.masks);
     }
     D.n_bonds = d->n_bonds;
     UP(bij.data(), bij.size(), &D.bond_ij);
@@ -760,6 +761,8 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
   }
   D.f32.ewald_beta = (float)D.ewald_beta;
   s->seg = segment_config(D, 0);
+  rows.charges_in_smem = s->seg.rows.charges_in_smem;
+  s->seg.rows = rows;
   if (s->seg.smem > kMaxSmem) {
     grp_destroy_system(s);
     return fail(GRP_ENOTIMPL, "system of %d atoms needs %zu bytes of shared memory per replica", n, s->seg.smem);
@@ -1069,7 +1072,7 @@ extern "C" grp_status grp_batch_create(grp_replicas *const *runs, int32_t n_runs
   for (int i = 0; i < n_runs; ++i) {
     const grp_replicas *r = runs[i];
     b->threads = std::max(b->threads, r->sys->seg.threads);
-    b->smem = std::max(b->smem, r->sys->seg.smem);
+    b->smem = std::max(b->smem, r->sys->seg.batch_smem);
     for (int k = 0; k < r->R; ++k) { units.push_back(make_uint2(i, k)); bunits.push_back(make_uint2(i, k)); }
     for (int j = 0; j < r->sys->dev.n_obs; ++j) gunits.push_back(make_uint2(i, j));
   }
@@ -1128,7 +1131,6 @@ static void fill_args(grp_batch *b, int k, const RunTick *ticks) {
     a.pairs_in_smem = r->sys->seg.pairs_in_smem;
     a.noise_batch = r->sys->seg.noise_batch;
     a.lean = r->sys->seg.lean;
-    a.charges_in_smem = r->sys->seg.charges_in_smem;
     b->h_args[i] = a;
   }
   for (int i = 0; i < nr; ++i) {

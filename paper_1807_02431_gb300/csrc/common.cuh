@@ -53,29 +53,19 @@ struct SysDev {
   const double *sd_d;      // [n] noise amplitudes sqrt((1 - c1^2) kT m) of the O step (large systems)
   const float *sd_f;
   int n_pairs;             // explicit non-excluded pair list (i | j << 16), i < j
-  const uint32_t *pairs;
   int n_items;             // force-field work items, (kind << 28) | index, each kind padded to a
-  const uint32_t *items;   // multiple of 32 entries so that a warp runs a single kind of item
+                           // multiple of 32 entries so that a warp runs a single kind of item
+  const uint32_t *pairs;
+  const uint32_t *items;
   // Tiled nonbonded path (tiled = 1): atoms in tiles of 32; every tile pair I <= J with, per lane
   // of tile I, a 32-bit mask of the atoms of tile J it interacts with (exclusions, padding and, on
   // the diagonal, i != j removed); the explicit pair items are then not in the item table.
   int tiled;
   int n_tiles, n_tile_pairs;
+  int use_rows;                // neighbour rows (RowsDev) in place of the Verlet list's pairs
   const uint32_t *tile_pairs;  // I | J << 16
   const uint32_t *tile_masks;  // [n_tile_pairs][32]
-  // Neighbour rows (rows.cuh): for tiles I and J and atom i = 32 I + lane, the atoms of J on i's row: not excluded, and
-  // of i < j with i + j odd or i > j with i + j even
-  int use_rows;
-  const uint32_t *row_masks;   // [n_tiles][n_tiles][32]
-  // soft springs as static rows: partners, 0xFFFF for none; strengths and lengths of the same places; the remaining
-  // bonds by index
-  const int *spring_rows;      // [n_tiles] rows of a tile's longest atom
-  const ushort4 *spring_j;     // [rows / 4][n]
-  const float4 *spring_f;      // [rows / 4][n][2] (k, r0, k, r0)
-  int n_stiff;
-  const int *stiff;
   double cutoff2;          // 0: no cutoff
-  float cutoff2_f;
   int coulomb_rf;          // Coulomb model: 0 dielectric eps = 4r, 1 reaction field (eps_r = 1),
                            // 2 periodic: Ewald real space on pairs plus particle mesh Ewald
   int gb;                  // 1: Generalized Born (OBC II) implicit solvent
@@ -84,15 +74,15 @@ struct SysDev {
   const double *con_len;
   double con_tol;          // relative tolerance of SHAKE / RATTLE
   int con_max_iter;
-  const unsigned char *con_atom;  // [n] 1 for atoms of a constraint
   int n_cgroups;           // connected groups of constraints (independent of each other)
+  const unsigned char *con_atom;  // [n] 1 for atoms of a constraint
   const int *cgroup_off;   // [n_cgroups + 1] into cgroup_cons and cgroup_atoms_off
   const int *cgroup_cons;  // constraint indices of each group, ascending
   const int *cgroup_aoff;  // [n_cgroups + 1] into cgroup_atoms
   const int *cgroup_atoms; // atoms of each group
   int n_gb_pairs;          // every pair i < j (i | j << 16) (systems of the item table)
-  const uint32_t *gb_pairs;
   int n_gb_xpairs;         // the excluded pairs i < j (systems with Verlet lists, whose lists omit them)
+  const uint32_t *gb_pairs;
   const uint32_t *gb_xpairs;
   double gb_tau;           // k_e (1/eps_in - 1/eps_out)
   const double4 *gb_d;     // per atom (rho - 0.009, 1/rho, S (rho - 0.009), q)
@@ -136,6 +126,22 @@ struct SysDev {
   int n_obs;
   int obs_kind[kMaxObs];
   int obs_arg[kMaxObs][4];
+};
+
+// Neighbour rows (rows.cuh) of a system with use_rows: for tiles I and J and atom i = 32 I + lane, the atoms of J on
+// i's row: not excluded, and of i < j with i + j odd or i > j with i + j even.  Soft springs as static rows:
+// partners, 0xFFFF for none; strengths and lengths of the same places; the remaining bonds by index.  (An argument
+// of its own: the batched kernel, which keeps the pair list, holds SegArgs in shared memory, and every byte of it is
+// one less for a replica.)
+struct RowsDev {
+  const uint32_t *masks;       // [n_tiles][n_tiles][32]
+  const int *spring_rows;      // [n_tiles] rows of a tile's longest atom
+  const ushort4 *spring_j;     // [rows / 4][n]
+  const float4 *spring_f;      // [rows / 4][n][2] (k, r0, k, r0)
+  const int *stiff;
+  int n_stiff;
+  float cutoff2;
+  int charges_in_smem;         // the charges in an array of their own
 };
 
 // ------------------------------------------------------------------------------------------------

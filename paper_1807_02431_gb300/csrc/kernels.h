@@ -28,7 +28,6 @@ struct SegArgs {
   int pairs_in_smem;
   int noise_batch;           // steps of noise generated together (0: drawn inline per atom)
   int lean;                  // atom parameters read from the global table (large systems)
-  int charges_in_smem;       // the charges in an array of their own (neighbour rows)
   uint32_t *nbl;             // [R][nbl_cap] Verlet lists (systems with use_list), else null
   float4 *qref;              // [R][n] positions at the last list build
   int nbl_cap;
@@ -44,10 +43,11 @@ constexpr int kMaxThreadChoices = 4;
 struct SegConfig {
   int threads;
   size_t smem;
+  size_t batch_smem;  // of the batched kernel, which keeps no charge array
   int pairs_in_smem;
   int noise_batch;
   int lean;
-  int charges_in_smem;
+  RowsDev rows;  // systems with neighbour rows
   // smaller blocks for many replicas (item-table systems): choice[0] = threads, and how many blocks of each size
   // the device holds at once
   int n_choices;

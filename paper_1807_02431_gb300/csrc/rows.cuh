@@ -107,13 +107,13 @@ struct RowList {
 };
 
 // Builds the rows of one replica: every non-excluded pair closer than cutoff + skin, on one of its atoms' rows
-// (S.row_masks).  A warp takes a tile, tests the boxes of 32 partner tiles at once, and for each near one tests
+// (RowsDev::masks).  A warp takes a tile, tests the boxes of 32 partner tiles at once, and for each near one tests
 // the 16 atoms j that can be on the lane's row (even lanes the odd ones and the other way round: two
 // addresses for the whole warp), collecting a mask, and then writes the mask's atoms to the row.  (The pair-list
 // build rotated j over the lanes and wrote through warp ballots: 640k cycles a build on the 2,030-atom
 // ligand.)  False when a row or the blocks have no room (the caller then builds the pair form).  Called by every
 // thread of the block; `bins` is scratch of 128 words, `taken` one more.
-__device__ __forceinline__ bool build_rows(const SysDev &S, const State<PathMixed> &st, const float *boxes, uint32_t *pool, int cap, RowList &L,
+__device__ __forceinline__ bool build_rows(const SysDev &S, const RowsDev &W, const State<PathMixed> &st, const float *boxes, uint32_t *pool, int cap, RowList &L,
                            int *bins, int *taken) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, n = S.n;
   const RowPool R = row_pool(S, cap);
@@ -146,7 +146,7 @@ __device__ __forceinline__ bool build_rows(const SysDev &S, const State<PathMixe
       }
       unsigned todo = __ballot_sync(0xffffffffu, near);
       auto mask_of = [&](unsigned b) {
-        return S.row_masks[((size_t)I * S.n_tiles + (e0 + __ffs(b) - 1)) * 32 + lane];
+        return W.masks[((size_t)I * S.n_tiles + (e0 + __ffs(b) - 1)) * 32 + lane];
       };
       uint32_t next_mask = todo ? mask_of(todo) : 0u;
       for (; todo; todo &= todo - 1) {
@@ -362,7 +362,6 @@ template <int kRF, bool kE>
 struct ListRow {
   using P = PathMixed;
   using T = float;
-  const SysDev &S;
   const Pos<P> &pos;
   const Params<P> &par;
   const AccMixed &acc;
@@ -373,9 +372,9 @@ struct ListRow {
   typename Pos<P>::At pi;
   T ash, ase, aqc;
   RowForce sum;
-  __device__ __forceinline__ ListRow(const SysDev &S_, const Pos<P> &pos_, const Params<P> &par_, const AccMixed &a,
+  __device__ __forceinline__ ListRow(float cutoff2, const Pos<P> &pos_, const Params<P> &par_, const AccMixed &a,
                                      long long &e, int *er)
-      : S(S_), pos(pos_), par(par_), acc(a), e_fix(e), err(er), cut2(S_.cutoff2_f) {}
+      : pos(pos_), par(par_), acc(a), e_fix(e), err(er), cut2(cutoff2) {}
   __device__ __forceinline__ void begin(int at) {
     i = at;
     pi = pos.at(at);
@@ -434,24 +433,24 @@ struct ListRow {
 // strengths and lengths beside them; the host gives each spring to the atom with the shorter row, so the rows of
 // all atoms are about equally long.  A warp takes a tile; the next block's places are loaded ahead, across tiles.
 // Stiff bonds, whose length needs double-single arithmetic, stay in a list of their own.
-__device__ __forceinline__ void spring_rows(const SysDev &S, const Pos<PathMixed> &pos, const Params<PathMixed> &par,
+__device__ __forceinline__ void spring_rows(const SysDev &S, const RowsDev &W, const Pos<PathMixed> &pos, const Params<PathMixed> &par,
                                             const AccMixed &acc, bool want_e, long long &e_fix, int *err) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, n = S.n;
   for (int I = warp; I < S.n_tiles; I += nwarps) {
-    const int i = I * 32 + lane, nb = (S.spring_rows[I] + 3) >> 2, ic = i < n ? i : n - 1;
+    const int i = I * 32 + lane, nb = (W.spring_rows[I] + 3) >> 2, ic = i < n ? i : n - 1;
     if (nb == 0) continue;
     RowForce sum;
     const float4 qi = pos.qh[ic];  // the high words suffice, as in bond_eval
-    ushort4 next = __ldg(S.spring_j + ic);
-    float4 nka = __ldg(S.spring_f + 2 * (size_t)ic), nkb = __ldg(S.spring_f + 2 * (size_t)ic + 1);
+    ushort4 next = __ldg(W.spring_j + ic);
+    float4 nka = __ldg(W.spring_f + 2 * (size_t)ic), nkb = __ldg(W.spring_f + 2 * (size_t)ic + 1);
     for (int b = 0; b < nb; ++b) {
       const ushort4 j4 = next;
       const float4 ka = nka, kb = nkb;
       const size_t at = (size_t)b * n + ic;
       if (b + 1 < nb) {
-        next = __ldg(S.spring_j + at + n);
-        nka = __ldg(S.spring_f + 2 * (at + n));
-        nkb = __ldg(S.spring_f + 2 * (at + n) + 1);
+        next = __ldg(W.spring_j + at + n);
+        nka = __ldg(W.spring_f + 2 * (at + n));
+        nkb = __ldg(W.spring_f + 2 * (at + n) + 1);
       }
       const float k[4] = {ka.x, ka.z, kb.x, kb.z}, r0[4] = {ka.y, ka.w, kb.y, kb.w};
       const int J[4] = {j4.x, j4.y, j4.z, j4.w};
@@ -481,8 +480,8 @@ __device__ __forceinline__ void spring_rows(const SysDev &S, const Pos<PathMixed
     }
     if (i < n) sum.flush(acc, i);
   }
-  for (int t = threadIdx.x; t < S.n_stiff; t += blockDim.x) {
-    const int b = S.stiff[t];
+  for (int t = threadIdx.x; t < W.n_stiff; t += blockDim.x) {
+    const int b = W.stiff[t];
     const int2 ij = S.bond_ij[b];
     bond_term<PathMixed>(pos, par, b, ij.x, ij.y, acc, want_e, e_fix, err);
   }

@@ -296,7 +296,7 @@ __device__ int build_list(const SysDev &S, const State<P> &st, float *boxes, uin
 }
 
 // The Verlet list of one replica in rows (or in pairs, when a row or the blocks had no room).
-__device__ __forceinline__ void build_row_list(const SysDev &S, const State<PathMixed> &st, float *boxes, uint32_t *pool,
+__device__ __forceinline__ void build_row_list(const SysDev &S, const RowsDev &W, const State<PathMixed> &st, float *boxes, uint32_t *pool,
                                                int cap, RowList &L, float4 *qref, int *bins, int *cnt, int *err) {
   tile_boxes<PathMixed>(S, st, boxes);
   for (int at = threadIdx.x; at < S.n; at += blockDim.x) {
@@ -305,7 +305,7 @@ __device__ __forceinline__ void build_row_list(const SysDev &S, const State<Path
     qref[at] = make_float4(x[0], x[1], x[2], 0.f);
   }
   L.n_pairs = -1;
-  if (!build_rows(S, st, boxes, pool, cap, L, bins, cnt)) {
+  if (!build_rows(S, W, st, boxes, pool, cap, L, bins, cnt)) {
     L.n_pairs = build_list<PathMixed>(S, st, boxes, pool, cap, qref, cnt, err);
     __syncthreads();
   }
@@ -396,7 +396,7 @@ enum : int {
 // The single-run kernels are compiled for one model, which keeps one copy of the force passes and no
 // unused solvent code in the step loop.
 template <class P, int kMode, int kFF>
-__device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsigned char *smem) {
+__device__ __forceinline__ void segment_body(const SegArgs &a, const RowsDev &W, const int r, unsigned char *smem) {
   using T = typename P::T;
   const SysDev &S = a.S;
   const int kThreads = (int)blockDim.x;
@@ -423,7 +423,7 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
   constexpr int kRF = kFF == 4 ? 2 : (kFF >= 2 ? 0 : kFF);
   float *qcs = nullptr;  // the charges side by side (rows)
   if constexpr (kRows)
-    if (a.charges_in_smem) {
+    if (W.charges_in_smem) {
       qcs = (float *)ptr;
       ptr += (size_t)n * 4;
       for (int i = threadIdx.x; i < n; i += kThreads) qcs[i] = S.atom_f[i].z;
@@ -486,7 +486,7 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
   int err = 0;
   RowList rl{list, n, 0, 0, 0, -1};
   auto rebuild = [&](int *e) {
-    if constexpr (kRows) build_row_list(S, st, boxes, list, a.nbl_cap, rl, qref, reinterpret_cast<int *>(red), lcount, e);
+    if constexpr (kRows) build_row_list(S, W, st, boxes, list, a.nbl_cap, rl, qref, reinterpret_cast<int *>(red), lcount, e);
     else n_list = build_list<P>(S, st, boxes, list, a.nbl_cap, qref, lcount, e);
   };
   if constexpr (kRows) {
@@ -598,10 +598,10 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
     auto passes = [&](auto rf) {
       constexpr int R = decltype(rf)::value;
       if constexpr (kRows) {
-        spring_rows(S, pos, par, fa, sample, e_fix, &err);
+        spring_rows(S, W, pos, par, fa, sample, e_fix, &err);
         angle_dihedral_pass<P>(S, pos, par, fa, sample, e_fix, &err);
-        if (sample) visit_rows(rl, ListRow<R, true>(S, pos, par, fa, e_fix, &err));
-        else visit_rows(rl, ListRow<R, false>(S, pos, par, fa, e_fix, &err));
+        if (sample) visit_rows(rl, ListRow<R, true>(W.cutoff2, pos, par, fa, e_fix, &err));
+        else visit_rows(rl, ListRow<R, false>(W.cutoff2, pos, par, fa, e_fix, &err));
         return;
       }
       if (lean) bonded_pass<P>(S, pos, par, fa, sample, e_fix, &err);
@@ -671,10 +671,10 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const int r, unsi
 // kMaxThreads/kMinBlocks: blocks of up to 320 threads keep two resident per SM (256 replica blocks
 // on 152 SMs then run in one wave); larger systems use up to 512 threads, one block per SM.
 template <class P, int kMaxThreads, int kMinBlocks, int kMode, int kFF>
-__global__ void __launch_bounds__(kMaxThreads, kMinBlocks) ff_segment_kernel(const SegArgs a) {
+__global__ void __launch_bounds__(kMaxThreads, kMinBlocks) ff_segment_kernel(const SegArgs a, const RowsDev rows) {
   if (a.skip_if_exit && exit_seen_before(a)) return;
   extern __shared__ __align__(16) unsigned char smem[];
-  segment_body<P, kMode, kFF>(a, blockIdx.x, smem);
+  segment_body<P, kMode, kFF>(a, rows, blockIdx.x, smem);
 }
 
 // Batched segments: a persistent grid of blocks takes (run, replica) units from a queue sorted by
@@ -688,6 +688,8 @@ __global__ void __launch_bounds__(512, 1) ff_segment_batch_kernel(const SegArgs 
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ SegArgs sa;
   __shared__ int su;
+  // beside the replica's state, which takes the rest of the 227 KB for systems of 2,380 to 2,500 atoms
+  static_assert(sizeof(SegArgs) + 8 <= 1120, "a larger SegArgs takes the largest systems out of batches");
   for (;;) {
     if (threadIdx.x == 0) {
       // units of replicas beyond a run's n_active (a transient advances replica 0 alone, a finished
@@ -709,7 +711,7 @@ __global__ void __launch_bounds__(512, 1) ff_segment_batch_kernel(const SegArgs 
     int *dst = reinterpret_cast<int *>(&sa);
     for (int i = threadIdx.x; i < (int)(sizeof(SegArgs) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
     __syncthreads();
-    segment_body<P, kModeAny, -1>(sa, (int)un.y, smem);
+    segment_body<P, kModeAny, -1>(sa, RowsDev{}, (int)un.y, smem);
     __syncthreads();
   }
 }
@@ -957,8 +959,9 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
     c.noise_batch = nb = 0;
   }
   c.pairs_in_smem = ff_smem_bytes(S, 1, nb, c.lean) <= 160 * 1024 ? 1 : 0;
-  c.charges_in_smem = S.use_rows && ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean, 1) <= kMaxSmem;
-  c.smem = ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean, c.charges_in_smem);
+  c.rows.charges_in_smem = S.use_rows && ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean, 1) <= kMaxSmem;
+  c.smem = ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean, c.rows.charges_in_smem);
+  c.batch_smem = ff_smem_bytes(S, c.pairs_in_smem, nb, c.lean);
   c.n_choices = 1;
   c.choice[0] = c.threads;
   if (!S.tiled && S.coulomb_rf != 2 && threads_hint <= 0 && c.smem <= kMaxSmem) {
@@ -990,7 +993,7 @@ static cudaError_t launch_ff_p(const SegArgs &a, const SegConfig &c, cudaStream_
   auto kern = ff_kernel<P>(a.S, threads);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);
   if (e != cudaSuccess) return e;
-  kern<<<a.n_active, threads, c.smem, st>>>(a);
+  kern<<<a.n_active, threads, c.smem, st>>>(a, c.rows);
   return cudaGetLastError();
 }
 
@@ -1019,7 +1022,6 @@ cudaError_t launch_segment(const SegArgs &a0, const SegConfig &c, cudaStream_t s
   a.pairs_in_smem = c.pairs_in_smem;
   a.noise_batch = c.noise_batch;
   a.lean = c.lean;
-  a.charges_in_smem = c.charges_in_smem;
   if (a.n_active <= 0) return cudaSuccess;
   if (a.S.potential == GRP_POT_DOUBLE_WELL_2D) {
     return launch_dw(a, st);

@@ -82,3 +82,31 @@ def test_dense_clumps(B, side):
     s.q0, s.p0 = x, W.maxwell_boltzmann(s.mass, s.kT, 3, rng)
     for a, b in zip(*_pair(B, s, 2, 40, 10)):
         assert np.array_equal(a, b)
+
+
+def _gas(n, cutoff, seed=3):
+    """n weakly charged beads on a lattice of 0.9 nm."""
+    rng = np.random.default_rng(seed)
+    m = int(np.ceil(n ** (1 / 3)))
+    x = np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n] * 0.9
+    s = W.System(name="gas", n_atoms=n, dim=3, potential=W.POT_FORCE_FIELD, mass=np.full(n, 12.0), kT=0.1, gamma=1.0,
+                 dt=0.002, sigma=np.full(n, 0.3), epsilon=np.full(n, 0.1), charge=rng.normal(0, 0.1, n),
+                 excl=np.zeros((0, 2), np.int32), cutoff=cutoff, coulomb_k=W.COULOMB_K, cv_kind=W.CV_COM_DISTANCE,
+                 cv_params=(1.0,), groups=[[0], [1]], observables=[(W.OBS_POTENTIAL, ()), (W.OBS_KINETIC, ())])
+    s.q0, s.p0 = x, W.maxwell_boltzmann(s.mass, s.kT, 3, rng)
+    return s
+
+
+@pytest.mark.parametrize("prec,n,cutoff", [(1, 2380, 1.2), (1, 2381, 1.2), (1, 2393, 1.2), (1, 2394, 1.2), (1, 2484, 1.2),
+                                           (1, 2504, 0.0), (0, 2381, 1.2), (0, 2400, 0.0)])
+def test_largest_batched_systems(B, prec, n, cutoff):
+    """The largest systems that a batch can hold beside its 1,120 bytes of launch arguments, on both precisions, with
+    and without lists, and the sizes at which the single run's charge array stops fitting (2,393): accepted, and equal to
+    the run alone."""
+    s = _gas(n, cutoff)
+    sysh = B.grp_create_system(s, B.GRP_MIXED if prec else B.GRP_FP64)
+    alone, run = (B.grp_init_replicas(sysh, 1, SEED, s.q0[None], s.p0[None], per_replica=True) for _ in range(2))
+    B.grp_step_k(alone, 3, 1)
+    B.grp_batch_step_k(B.grp_batch_create([run]), 3, 1)
+    for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(run)[:3]):
+        assert np.array_equal(a, b)
