@@ -88,6 +88,7 @@ struct grp_replicas {
   uint32_t *nbl = nullptr;  // [R][nbl_cap] Verlet lists
   float4 *qref = nullptr;   // [R][n]
   int nbl_cap = 0;
+  int use_rows = 0;  // neighbour rows, where the system has them and the first configuration's fit
   long long t_global = 0, t_phase = 0;
   // shard of a run sharded over processes: global index of replica 0 and the run's replica count
   // (rep0 = 0, n_global = R for a set that is the whole run)
@@ -851,6 +852,7 @@ extern "C" grp_status grp_init_replicas(grp_system *s, int32_t n_replicas, uint6
     const double lc2 = (double)D.list_cut2;
     const bool per = D.coulomb_rf == 2;
     size_t cnt = 0;
+    std::vector<int> row(n, 0);  // of the neighbour rows: the lower atom's when the sum is odd
     for (int i = 0; i < n; ++i)
       for (int j = i + 1; j < n; ++j) {
         if (s->excl[(size_t)i * n + j]) continue;
@@ -860,8 +862,11 @@ extern "C" grp_status grp_init_replicas(grp_system *s, int32_t n_replicas, uint6
           if (per) dx -= D.box[x] * std::nearbyint(dx * D.ibox[x]);
           d2 += dx * dx;
         }
-        cnt += d2 < lc2;
+        if (!(d2 < lc2)) continue;
+        ++cnt;
+        ++row[((i + j) & 1) ? i : j];
       }
+    r->use_rows = D.use_rows && *std::max_element(row.begin(), row.end()) <= kRowPartners;
     const size_t all = (size_t)n * (n - 1) / 2;
     // at least 65,536 entries (every pair, for systems of up to ~360 atoms, whose density may still
     // change a lot: ions condensing in a periodic box), + the padding of the warps' partly filled chunks
@@ -941,6 +946,7 @@ static SegArgs seg_args(grp_replicas *r, int k, int t_gr, int n_active) {
   a.nbl = r->nbl;
   a.qref = r->qref;
   a.nbl_cap = r->nbl_cap;
+  a.S.use_rows = r->use_rows;
   a.gb_glob = r->gb_glob;
   a.gb_gr = r->gb_gr;
   a.gb_gr_stride = r->gb_gr_stride;

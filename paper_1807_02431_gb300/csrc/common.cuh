@@ -31,6 +31,9 @@ constexpr float kSoftBond = 1.0e4f;
 // warps (1,024 atoms, 40 replicas x 60 steps, 3.7 -> 2.9 ms; 2,030 atoms 11.5 -> 9.6 with 200).  With seven tiles (220
 // atoms in a periodic box) rows were slower than the pair list.
 constexpr int kRowsMinAtoms = 1024;
+// Partners that a row holds.  A replica set whose first configuration has longer rows keeps the pair list (globules of
+// 1,024 atoms with a cutoff of 1.2 nm: from about 50 atoms per nm^3 on).
+constexpr int kRowPartners = 256;
 
 // Scalars of a system rounded to FP32 on the host, for the pair loops of the mixed path: a conversion in the kernel
 // is an instruction at the FP64 pipe's rate, and under register pressure the compiler repeats it where the value is

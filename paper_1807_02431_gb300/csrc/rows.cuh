@@ -12,7 +12,11 @@
 // largest displacement requires (22 % fewer partners, but the rebuild grew by half: 268 ms), forces kept in the
 // accumulators to save their array (256 ms), lists rebuilt in a function of its own (290 ms).  Smaller, periodic and
 // solvated systems keep the pair list: 220 atoms in a periodic box took 26.9 ms against 24.6 (seven tiles are too few
-// rows for sixteen warps), the solvated ligand 380 against 325 (its passes spill).
+// rows for sixteen warps), the solvated ligand 380 against 325 (its passes spill).  So do replica sets whose rows would
+// be longer than kRowPartners, and a replica that outgrows its rows on the way takes the pair list for the rest of the
+// launch (segment.cu).  As rows of one pair each they took three times the pair list's time: globules at 100 atoms per
+// nm^3 within 1.2 nm, 152 replicas x 20 steps, 1,024 atoms 5.5 -> 16.7 ms, 2,030 atoms 13.7 -> 39.4; at 40 per
+// nm^3, whose rows fit, rows take 2.7 against 3.1 and 6.4 against 7.0 ms.
 #pragma once
 #include "state.cuh"
 
@@ -69,15 +73,13 @@ struct RowForce {
 
 // ---- the Verlet list of one replica
 // Its memory is a pool of `cap` 32-bit words.
-// Row form: the rows are sorted by length and taken 32 at a time, so that the 32 rows of a warp are about equally long; such a group holds its partners in blocks
-// of 4 x 32 16-bit places, [block][lane][4], so that a lane's next four partners are one 8-byte load and a
+// The rows are sorted by length and taken 32 at a time, so that the 32 rows of a warp are about equally long; such a
+// group holds its partners in blocks of 4 x 32 16-bit places, [block][lane][4], so that a lane's next four partners are one 8-byte load and a
 // warp's are contiguous.  Blocks are worked off in chunks of up to `chunk` blocks of one group, so that the
 // warps of the block get equal shares.  Tables at the end of the pool: the rows in order and their lengths,
 // the groups' first blocks, and the chunks (group | blocks << 16 | first block in the group << 20, first block).
-// Pair form (n_pairs >= 0; only when a row outgrew its place at the last build): i | j << 16 per word,
-// 0xFFFFFFFF for none.
 // While rows are built, those of a tile grow together in pieces of eight places for each of its 32 atoms
-// ([lane][8], 512 bytes), taken one by one from the rest of the pool, up to 32 pieces (256 partners) a tile.
+// ([lane][8], 512 bytes), taken one by one from the rest of the pool, up to 32 pieces (kRowPartners) a tile.
 struct RowPool {
   int groups;  // of 32 rows
   int places;                // places of the blocks
@@ -103,7 +105,6 @@ struct RowList {
   const uint32_t *pool;
   int n, order, chunks;  // atoms, word offsets of the tables
   int n_chunks;
-  int n_pairs;
 };
 
 // Builds the rows of one replica: every non-excluded pair closer than cutoff + skin, on one of its atoms' rows
@@ -111,7 +112,7 @@ struct RowList {
 // the 16 atoms j that can be on the lane's row (even lanes the odd ones and the other way round: two
 // addresses for the whole warp), collecting a mask, and then writes the mask's atoms to the row.  (The pair-list
 // build rotated j over the lanes and wrote through warp ballots: 640k cycles a build on the 2,030-atom
-// ligand.)  False when a row or the blocks have no room (the caller then builds the pair form).  Called by every
+// ligand.)  False when a row or the blocks have no room (the caller then builds the pair list).  Called by every
 // thread of the block; `bins` is scratch of 128 words, `taken` one more.
 __device__ __forceinline__ bool build_rows(const SysDev &S, const RowsDev &W, const State<PathMixed> &st, const float *boxes, uint32_t *pool, int cap, RowList &L,
                            int *bins, int *taken) {
@@ -175,7 +176,7 @@ __device__ __forceinline__ bool build_rows(const SysDev &S, const RowsDev &W, co
           int id = 0;
           if (lane == 0) id = atomicAdd(taken, 1);
           id = __shfl_sync(0xffffffffu, id, 0);
-          if (have >= 32 || id >= R.pieces) { over = 1; break; }
+          if (have >= kRowPartners / 8 || id >= R.pieces) { over = 1; break; }
           if (lane == have) mine = id;
           ++have;
         }
@@ -294,18 +295,16 @@ __device__ __forceinline__ bool build_rows(const SysDev &S, const RowsDev &W, co
 
 // The rows of a replica, shared out over the warps of the block chunk by chunk.  The visitor's begin(i),
 // batch(partners, count) -- four places at a time, the first `count` of them filled (count <= 0: none) -- and
-// end(any) are called by whole warps.  In pair form a unit is 32 pairs, each a row of one.  The
-// next chunk's row and first partners are loaded ahead.
+// end(any) are called by whole warps.  The next chunk's row and first partners are loaded ahead.
 template <class V>
 __device__ __forceinline__ void visit_rows(const RowList &L, V &&v) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const bool pairs = L.n_pairs >= 0;
-  const int units = pairs ? (L.n_pairs + 31) >> 5 : L.n_chunks;
+  const int units = L.n_chunks;
   const uint2 *table = reinterpret_cast<const uint2 *>(L.pool + L.chunks);
   const ushort4 *blocks = reinterpret_cast<const ushort4 *>(L.pool) + lane;
   // loaded ahead: the table entry two units, the row and its first partners one unit
   const uint2 *order = reinterpret_cast<const uint2 *>(L.pool + L.order);
-  auto entry = [&](int u) { return u < units && !pairs ? table[u] : make_uint2(0u, 0u); };
+  auto entry = [&](int u) { return u < units ? table[u] : make_uint2(0u, 0u); };
   struct Unit {
     int i, cnt, nb, block;
     ushort4 j;
@@ -313,22 +312,13 @@ __device__ __forceinline__ void visit_rows(const RowList &L, V &&v) {
   auto load = [&](int u, uint2 e) {
     Unit x{0, 0, 0, 0, make_ushort4(0, 0, 0, 0)};
     if (u >= units) return x;
-    if (pairs) {
-      const int pos = u * 32 + lane;
-      const uint32_t w = pos < L.n_pairs ? L.pool[pos] : 0xFFFFFFFFu;
-      x.nb = 1;
-      x.cnt = w != 0xFFFFFFFFu ? 1 : 0;
-      x.i = x.cnt ? (int)(w & 0xFFFFu) : 0;
-      x.j.x = (unsigned short)(w >> 16);
-    } else {
-      const int pos = 32 * (int)(e.x & 0xFFFFu) + lane;
-      const uint2 w = pos < L.n ? order[pos] : make_uint2(0u, 0u);
-      x.block = (int)e.y;
-      x.j = blocks[(size_t)x.block * 32];
-      x.nb = (int)((e.x >> 16) & 15u);
-      x.i = (int)w.x;
-      x.cnt = (int)w.y - 4 * (int)(e.x >> 20);
-    }
+    const int pos = 32 * (int)(e.x & 0xFFFFu) + lane;
+    const uint2 w = pos < L.n ? order[pos] : make_uint2(0u, 0u);
+    x.block = (int)e.y;
+    x.j = blocks[(size_t)x.block * 32];
+    x.nb = (int)((e.x >> 16) & 15u);
+    x.i = (int)w.x;
+    x.cnt = (int)w.y - 4 * (int)(e.x >> 20);
     return x;
   };
   Unit next = load(warp, entry(warp));

@@ -295,20 +295,16 @@ __device__ int build_list(const SysDev &S, const State<P> &st, float *boxes, uin
   return c;
 }
 
-// The Verlet list of one replica in rows (or in pairs, when a row or the blocks had no room).
-__device__ __forceinline__ void build_row_list(const SysDev &S, const RowsDev &W, const State<PathMixed> &st, float *boxes, uint32_t *pool,
-                                               int cap, RowList &L, float4 *qref, int *bins, int *cnt, int *err) {
+// The Verlet list of one replica in rows; false when a row or the blocks had no room.
+__device__ __forceinline__ bool build_row_list(const SysDev &S, const RowsDev &W, const State<PathMixed> &st, float *boxes,
+                                               uint32_t *pool, int cap, RowList &L, float4 *qref, int *bins, int *cnt) {
   tile_boxes<PathMixed>(S, st, boxes);
   for (int at = threadIdx.x; at < S.n; at += blockDim.x) {
     float x[3];
     st.get_f32(at, x);
     qref[at] = make_float4(x[0], x[1], x[2], 0.f);
   }
-  L.n_pairs = -1;
-  if (!build_rows(S, W, st, boxes, pool, cap, L, bins, cnt)) {
-    L.n_pairs = build_list<PathMixed>(S, st, boxes, pool, cap, qref, cnt, err);
-    __syncthreads();
-  }
+  return build_rows(S, W, st, boxes, pool, cap, L, bins, cnt);
 }
 
 // Fixed-point sum (2^-40 units on the FP64 path, 2^-32 on the mixed path) to the path's precision,
@@ -484,10 +480,16 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const RowsDev &W,
   int n_list = 0;
 
   int err = 0;
-  RowList rl{list, n, 0, 0, 0, -1};
+  RowList rl{list, n, 0, 0, 0};
+  // neighbour rows until a build has no room for them; pairs from then on in this launch, so that a system that has
+  // outgrown the rows fails one build, not every one
+  bool in_rows = kRows;
   auto rebuild = [&](int *e) {
-    if constexpr (kRows) build_row_list(S, W, st, boxes, list, a.nbl_cap, rl, qref, reinterpret_cast<int *>(red), lcount, e);
-    else n_list = build_list<P>(S, st, boxes, list, a.nbl_cap, qref, lcount, e);
+    if constexpr (kRows) {
+      if (in_rows) in_rows = build_row_list(S, W, st, boxes, list, a.nbl_cap, rl, qref, reinterpret_cast<int *>(red), lcount);
+      if (in_rows) return;
+    }
+    n_list = build_list<P>(S, st, boxes, list, a.nbl_cap, qref, lcount, e);
   };
   if constexpr (kRows) {
     const RowPool rp = row_pool(S, a.nbl_cap);
@@ -600,7 +602,8 @@ __device__ __forceinline__ void segment_body(const SegArgs &a, const RowsDev &W,
       if constexpr (kRows) {
         spring_rows(S, W, pos, par, fa, sample, e_fix, &err);
         angle_dihedral_pass<P>(S, pos, par, fa, sample, e_fix, &err);
-        if (sample) visit_rows(rl, ListRow<R, true>(W.cutoff2, pos, par, fa, e_fix, &err));
+        if (!in_rows) list_pass<P, R>(S, pos, par, list, n_list, fa, sample, e_fix, &err);
+        else if (sample) visit_rows(rl, ListRow<R, true>(W.cutoff2, pos, par, fa, e_fix, &err));
         else visit_rows(rl, ListRow<R, false>(W.cutoff2, pos, par, fa, e_fix, &err));
         return;
       }

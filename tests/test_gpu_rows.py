@@ -110,3 +110,64 @@ def test_largest_batched_systems(B, prec, n, cutoff):
     B.grp_batch_step_k(B.grp_batch_create([run]), 3, 1)
     for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(run)[:3]):
         assert np.array_equal(a, b)
+
+
+def _globule(n, rho, seed=1):
+    """n weakly interacting beads at rho per nm^3, numbered along the lattice."""
+    rng = np.random.default_rng(seed)
+    a = rho ** (-1.0 / 3.0)
+    s = _gas(n, 1.2, seed)
+    m = int(np.ceil(n ** (1 / 3)))
+    s.q0 = np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n] * a + rng.uniform(-0.02, 0.02, (n, 3))
+    return dataclasses.replace(s, sigma=np.full(n, 0.6 * a), epsilon=np.full(n, 0.05), q0=s.q0, p0=s.p0, dt=0.001)
+
+
+@pytest.mark.parametrize("n,rho", [(1100, 60), (1100, 100), (2030, 100)])
+def test_dense_systems_keep_the_speed_of_pairs(B, n, rho):
+    """A set whose rows would be longer than their 256 places takes the pair list: as fast as the batched kernel,
+    which always does, within a third (through rows of one pair each it took three times as long)."""
+    import torch
+
+    s = _globule(n, rho)
+    q0, p0 = W.replica_states(s, 8, seed=6, spread=0.0005)
+    sysh = B.grp_create_system(s, B.GRP_MIXED)
+    alone, run = (B.grp_init_replicas(sysh, 8, SEED, q0, p0, per_replica=True) for _ in range(2))
+    batch = B.grp_batch_create([run])
+    ms = []
+    for step in (lambda: B.grp_step_k(alone, 20, 10), lambda: B.grp_batch_step_k(batch, 20, 10)):
+        t = []
+        for _ in range(4):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            step()
+            e[1].record()
+            torch.cuda.synchronize()
+            t.append(e[0].elapsed_time(e[1]))
+        ms.append(min(t))
+    assert ms[0] <= 1.33 * ms[1]
+    for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(run)[:3]):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("hub", [400, 600])
+def test_rows_outgrown_by_one_replica(B, hub):
+    """Replica 0, whose configuration decides, is a sparse gas; in replica 1 `hub` beads sit on a sphere of 1.3 nm around
+    one (a row of 200 partners, which fits, or of 300, which does not): that replica goes on in pairs."""
+    s = _gas(1100, 1.2)
+    s = dataclasses.replace(s, epsilon=np.zeros(1100), charge=s.charge * 0.1, q0=s.q0, p0=s.p0)
+    q1 = s.q0.copy() + 20.0
+    z = (2.0 * np.arange(hub) + 1.0) / hub - 1.0  # evenly: equal bands, the golden angle apart
+    phi = np.arange(hub) * np.pi * (3.0 - np.sqrt(5.0))
+    q1[0] = 0.0
+    q1[1:hub + 1] = 1.3 * np.stack([np.sqrt(1 - z * z) * np.cos(phi), np.sqrt(1 - z * z) * np.sin(phi), z], -1)
+    d = np.linalg.norm(q1[:, None] - q1[None], axis=-1) < 1.4
+    row0 = sum(d[0, j] for j in range(1, 1100) if j % 2)
+    assert (row0 > 256) == (hub > 512) and np.triu(d, 1).sum() < 65536
+    q0, p0 = np.stack([s.q0, q1, s.q0]), np.stack([s.p0] * 3)
+    sysh = B.grp_create_system(s, B.GRP_MIXED)
+    alone, run = (B.grp_init_replicas(sysh, 3, SEED, q0, p0, per_replica=True) for _ in range(2))
+    for k in (1, 40):
+        B.grp_step_k(alone, k, 10)
+        B.grp_batch_step_k(B.grp_batch_create([run]), k, 10)
+        for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(run)[:3]):
+            assert np.array_equal(a, b)
