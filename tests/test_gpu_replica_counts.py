@@ -1,5 +1,7 @@
 """Kernels whose launch shape follows the number of replicas: the double well's groups of replicas per block, and
 the block sizes of item-table systems, single and batched, against the FP64 oracle or a set of another size."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -88,4 +90,45 @@ def test_batched_block_sizes_give_the_same_bits(B, n_runs):
         alone = B.grp_init_replicas(sysh, R, SEED + i, q0, p0, per_replica=True)
         B.grp_step_k(alone, k, 5)
         for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(runs[i])[:3]):
+            assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("make", ["chain_h22", "chain_h30", "rf40", "cutoff40", "chain60", "solvated40"])
+def test_kernel_variants_give_the_same_bits(B, make, prec):
+    """Systems of more than 320 items, whose large sets run another instantiation of the kernel than the small ones: the
+    first replicas are the small set's bit for bit."""
+    s = {"chain_h22": lambda: W.chain_h(22), "chain_h30": lambda: W.chain_h(30),
+         "rf40": lambda: dataclasses.replace(W.chain(40), cutoff=1.0, coulomb_mode=W.COULOMB_REACTION_FIELD),
+         "cutoff40": lambda: dataclasses.replace(W.chain(40), cutoff=1.0), "chain60": lambda: W.chain(60),
+         "solvated40": lambda: W.solvated(W.chain(40))}[make]()
+    small, k = 4, 24
+    q0, p0 = W.replica_states(s, 700, seed=9, spread=0.002)
+    sysh = B.grp_create_system(s, B.GRP_FP64 if prec == "fp64" else B.GRP_MIXED)
+    out = []
+    for n in (small, 200, 400, 700):
+        rep = B.grp_init_replicas(sysh, n, SEED, q0[:n], p0[:n], per_replica=True)
+        B.grp_step_k(rep, k, 4)
+        out.append([x[:small] for x in B.grp_get_state(rep)[:3]])
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("make", ["chain10", "chain40", "rf22", "rf40", "alkane5"])
+@pytest.mark.parametrize("n_runs", [1, 100])
+def test_batches_give_the_bits_of_runs_alone(B, make, prec, n_runs):
+    """Batches of small systems on both precisions, with and without the reaction field: up to 400 units."""
+    rf = lambda n: dataclasses.replace(W.chain(n), cutoff=1.0, coulomb_mode=W.COULOMB_REACTION_FIELD)
+    s = {"chain10": lambda: W.chain(10), "chain40": lambda: W.chain(40), "rf22": lambda: rf(22), "rf40": lambda: rf(40),
+         "alkane5": lambda: W.alkane(5)}[make]()
+    R, k = 4, 24
+    q0, p0 = W.replica_states(s, R, seed=9, spread=0.002)
+    sysh = B.grp_create_system(s, B.GRP_FP64 if prec == "fp64" else B.GRP_MIXED)
+    alone, *runs = (B.grp_init_replicas(sysh, R, SEED, q0, p0, per_replica=True) for _ in range(n_runs + 1))
+    B.grp_step_k(alone, k, 4)
+    B.grp_batch_step_k(B.grp_batch_create(runs), k, 4)
+    for r in (runs[0], runs[-1]):
+        for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(r)[:3]):
             assert np.array_equal(a, b)
