@@ -8,6 +8,7 @@
 // = 1/2;  dE/d eps_ij = 4 (s^12 - s^6), d eps_ij / d eps_i = sqrt(eps_j) / (2 sqrt(eps_i)).  Per
 // dihedral term, dE/dk = 1 + cos(n phi - delta).  The sums use the 2^-40 fixed point of the FP64
 // force path, so the result does not depend on the order in which threads add their terms.
+#include <algorithm>
 #include <cfloat>
 
 #include "dual.cuh"
@@ -446,8 +447,11 @@ size_t adjoint_smem_bytes(const SysDev &S, int n_terms, int ck) {
          State<PathF64>::bytes(S.n, true) + 32;
 }
 
-template <class P>
-__global__ void __launch_bounds__(256) adjoint_kernel(const AdjArgs a) {
+// kMinBlocks: the mixed path's integer conversions take 115 registers where the compiler is free, two blocks per SM; bounded
+// to 80, three fit, each a little slower (22 beads, k = 50: 256 replicas 1,124 us against 1,146; 400 replicas, which
+// then take one wave instead of two, 1,904 against 1,326).  The FP64 path takes 116 either way.
+template <class P, int kMinBlocks>
+__global__ void __launch_bounds__(256, kMinBlocks) adjoint_kernel(const AdjArgs a) {
   using Tr = AdjointTraits<P>;
   using TP = typename Tr::TP;
   using T = typename P::T;
@@ -554,9 +558,17 @@ cudaError_t launch_adjoint(const AdjArgs &a, int n_rep, cudaStream_t st) {
   if (a.S.potential != GRP_POT_FORCE_FIELD || a.S.tiled) return cudaErrorInvalidValue;
   const size_t smem = adjoint_smem_bytes(a.S, a.n_terms, a.ck);
   if (smem > kMaxSmem) return cudaErrorInvalidValue;
-  auto kern = a.S.precision == GRP_FP64 ? adjoint_kernel<PathF64> : adjoint_kernel<PathMixed>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  // three blocks per SM where that saves a wave
+  const int per_sm = (int)((228 * 1024) / (smem + 1024));
+  const int two = sms * std::max(1, std::min(2, per_sm)), three = sms * std::max(1, std::min(3, per_sm));
+  const bool fewer = (n_rep + three - 1) / three < (n_rep + two - 1) / two;
+  auto kern = a.S.precision == GRP_FP64 ? adjoint_kernel<PathF64, 2>
+                                        : (fewer ? adjoint_kernel<PathMixed, 3> : adjoint_kernel<PathMixed, 2>);
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   kern<<<n_rep, 256, smem, st>>>(a);
   return cudaGetLastError();
 }

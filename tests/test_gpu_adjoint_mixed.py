@@ -94,3 +94,47 @@ def test_mixed_adjoint_full_launch(B):
     L64, _, _, _, _ = _adjoint(B, B.GRP_FP64, s, q0, p0, 1000, 100, lo)
     assert np.all(np.isfinite(g32)) and np.all(np.isfinite(q32)) and np.all(np.isfinite(p32))
     assert abs(L32 - L64) < 1e-3 * abs(L64)
+
+
+def test_mixed_adjoint_keeps_three_replicas_per_sm(B):
+    """Three blocks of the mixed adjoint fit on an SM, so three replicas per SM take less than 1.5 times as long as two
+    (as a second wave of blocks they took 1.7 times as long)."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    s = W.chain_gradient(22)
+    sysh = B.grp_create_system(s, B.GRP_MIXED)
+    grad = torch.empty(B.grp_param_count(sysh), dtype=torch.float64, device="cuda")
+    ms = []
+    for R in (2 * sms, 3 * sms):
+        q0, p0 = W.replica_states(s, R, seed=3, spread=0.002)
+        rep = B.grp_init_replicas(sysh, R, SEED, q0, p0, per_replica=True)
+        t = []
+        for _ in range(5):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            B.grp_adjoint_segment(rep, 50, s.t_gr, 25, 4, d_grad_theta=grad)
+            e[1].record()
+            torch.cuda.synchronize()
+            t.append(e[0].elapsed_time(e[1]))
+        ms.append(min(t))
+    assert ms[1] < 1.5 * ms[0]
+
+
+@pytest.mark.parametrize("n", [10, 22, 33])
+def test_mixed_adjoint_of_large_and_small_sets(B, n):
+    """Sets that run three replicas per SM and sets that run two: the same gradients of the first replicas (of their
+    share of the loss, 1 / R: powers of two, so that it scales them exactly)."""
+    import torch
+
+    s = W.chain_gradient(n)
+    sysh = B.grp_create_system(s, B.GRP_MIXED)
+    q0, p0 = W.replica_states(s, 2048, seed=3, spread=0.002)
+    out = []
+    for R in (4, 256, 512, 1024, 2048):
+        rep = B.grp_init_replicas(sysh, R, SEED, q0[:R], p0[:R], per_replica=True)
+        gq, gp = (torch.empty(R, n, 3, dtype=torch.float64, device="cuda") for _ in range(2))
+        B.grp_adjoint_segment(rep, 40, s.t_gr, 20, 4, d_grad_q0=gq, d_grad_p0=gp)
+        out.append((R * gq[:4].cpu().numpy(), R * gp[:4].cpu().numpy()))
+    for other in out[1:]:
+        assert np.array_equal(out[0][0], other[0]) and np.array_equal(out[0][1], other[1])
