@@ -52,6 +52,8 @@ struct SegConfig {
   // the device holds at once
   int n_choices;
   int choice[kMaxThreadChoices], slots[kMaxThreadChoices];
+  int sms;
+  double crowding;  // a wave of p blocks per SM takes p^crowding of the time of one block per SM
 };
 
 // Largest dynamic shared memory of one block on sm_103a.

@@ -1,9 +1,10 @@
 // Fused segment kernels: k BAOAB steps of Eq. 1 per replica with the replica's state held on chip,
 // observable sampling every t_GR (Section 2.4.1) and the exit test at the end of the segment
-// (Section 3.3).  One thread block per replica for force-field systems; one thread per replica for
-// the analytic 2-D double well.
+// (Section 3.3).  One thread block per replica for force-field systems; blocks of one, four or sixteen replicas
+// for the analytic 2-D double well.
+#include <algorithm>
 #include <cfloat>
-
+#include <cmath>
 #include <type_traits>
 
 #include "forcefield.cuh"
@@ -883,8 +884,8 @@ static auto ff_kernel(const SysDev &S, int threads) {
 
 // Blocks of the kernel that the device holds at once (0: unknown).
 template <class K>
-static int resident_blocks(K kern, int threads, size_t smem) {
-  int dev = 0, sms = 0, per_sm = 0;
+static int resident_blocks(K kern, int threads, size_t smem, int &sms) {
+  int dev = 0, per_sm = 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -898,7 +899,10 @@ static int resident_blocks(K kern, int threads, size_t smem) {
 // Block sizes of item-table systems.  One thread per item is the shortest step while every replica has a place on
 // the chip; a step is a chain of latencies, so with more replicas smaller blocks, of which more are resident, do
 // more steps per second.  Candidates from the default downwards, of which a launch takes the largest whose
-// blocks are all resident, or else the last: 512, 320, 192, 160 threads, and 64, 32 for systems of up to 128 items
+// blocks are all resident, or else the one of the least estimated time, waves x p^e for p blocks per SM (the last,
+// whatever its waves, was up to 25 % slower than the default: FP64 solvated 60 beads, 608 replicas x 10 steps, 7,070 us
+// with 512 threads, 8,640 with 160, 6,870 with the 320 now chosen; FP64 22 beads, 912 replicas, 468 us with 320, 523
+// with 160, 418 with 192): 512, 320, 192, 160 threads, and 64, 32 for systems of up to 128 items
 // (7 to 10 beads).  us per 100 steps, default -> chosen (mixed): 40 beads 256 replicas 466 -> 375 (512 -> 320
 // threads), 1,024 replicas 1,614 -> 1,185 (160); 60 beads 256 replicas 855 -> 756; 22 beads 400 replicas 303 -> 231
 // (192), 1,024 replicas 625 -> 485 (160); 24 atoms with constraints, 512 replicas 1,458 -> 856; solvated 22 beads,
@@ -917,10 +921,24 @@ static int thread_candidates(int threads, int out[kMaxThreadChoices]) {
   }
   return n;
 }
-static int choose_threads(const int *threads, const int *slots, int n, int units) {
-  for (int t = 0; t < n; ++t)
-    if (units <= slots[t]) return threads[t];
-  return threads[n - 1];
+// The exponent e: a system of 288 items (22 beads) takes 1.3 times as long with two blocks per SM as with one, of 1,856
+// (60 beads) 1.7 times; with constraints, one warp's chain is the step whatever runs beside it.
+static double crowding_of(int n_items, bool constraints) {
+  return constraints ? 0.0 : std::min(0.8, std::sqrt((double)n_items) / 55.0);
+}
+static int choose_threads(const SegConfig &c, int units) {
+  int best = 0;
+  double least = 1e300;
+  for (int t = 0; t < c.n_choices; ++t) {
+    if (units <= c.slots[t]) return c.choice[t];
+    const double cost = ((units + c.slots[t] - 1) / c.slots[t]) * std::pow((double)c.slots[t] / c.sms, c.crowding);
+    // (the smaller block of two of the same waves under constraints, the larger one otherwise)
+    if (c.crowding > 0.0 ? cost < least * (1.0 - 1e-9) : cost <= least) {
+      least = cost;
+      best = t;
+    }
+  }
+  return c.choice[best];
 }
 
 SegConfig segment_config(const SysDev &S, int threads_hint) {
@@ -969,9 +987,11 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
   c.choice[0] = c.threads;
   if (!S.tiled && S.coulomb_rf != 2 && threads_hint <= 0 && c.smem <= kMaxSmem) {
     c.n_choices = thread_candidates(c.threads, c.choice);
+    c.crowding = crowding_of(S.n_items, S.n_cons > 0);
     for (int t = 0; t < c.n_choices; ++t) {
-      c.slots[t] = S.precision == GRP_FP64 ? resident_blocks(ff_kernel<PathF64>(S, c.choice[t]), c.choice[t], c.smem)
-                                           : resident_blocks(ff_kernel<PathMixed>(S, c.choice[t]), c.choice[t], c.smem);
+      c.slots[t] = S.precision == GRP_FP64
+                       ? resident_blocks(ff_kernel<PathF64>(S, c.choice[t]), c.choice[t], c.smem, c.sms)
+                       : resident_blocks(ff_kernel<PathMixed>(S, c.choice[t]), c.choice[t], c.smem, c.sms);
       if (c.slots[t] == 0) c.n_choices = 1;  // nothing known: the default
     }
   }
@@ -979,19 +999,20 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
 }
 
 int batch_threads(int precision, int threads, size_t smem, int units) {
-  int cand[kMaxThreadChoices], slots[kMaxThreadChoices];
+  int cand[kMaxThreadChoices], sms = 0;
   const int n = thread_candidates(threads, cand);
   for (int t = 0; t < n; ++t) {
-    slots[t] = precision == GRP_FP64 ? resident_blocks(ff_segment_batch_kernel<PathF64>, cand[t], smem)
-                                     : resident_blocks(ff_segment_batch_kernel<PathMixed>, cand[t], smem);
-    if (slots[t] == 0) return threads;
+    const int slots = precision == GRP_FP64 ? resident_blocks(ff_segment_batch_kernel<PathF64>, cand[t], smem, sms)
+                                            : resident_blocks(ff_segment_batch_kernel<PathMixed>, cand[t], smem, sms);
+    if (slots == 0) return threads;
+    if (units <= slots) return cand[t];
   }
-  return choose_threads(cand, slots, n, units);
+  return cand[n - 1];
 }
 
 template <class P>
 static cudaError_t launch_ff_p(const SegArgs &a, const SegConfig &c, cudaStream_t st) {
-  const int threads = c.n_choices > 1 ? choose_threads(c.choice, c.slots, c.n_choices, a.n_active) : c.threads;
+  const int threads = c.n_choices > 1 ? choose_threads(c, a.n_active) : c.threads;
   if (threads < 32 || threads > 512 || threads % 32) return cudaErrorInvalidValue;
   auto kern = ff_kernel<P>(a.S, threads);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);

@@ -132,3 +132,34 @@ def test_batches_give_the_bits_of_runs_alone(B, make, prec, n_runs):
     for r in (runs[0], runs[-1]):
         for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(r)[:3]):
             assert np.array_equal(a, b)
+
+
+def _best_ms(step, n=5):
+    import torch
+
+    t = []
+    for _ in range(n):
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        e[0].record()
+        step()
+        e[1].record()
+        torch.cuda.synchronize()
+        t.append(e[0].elapsed_time(e[1]))
+    return min(t)
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+def test_twice_the_replicas_take_twice_as_long(B, prec):
+    """A set of two full waves takes two waves' time: twice the replicas that fill the chip in two blocks per SM take at
+    most 1.15 times twice as long (in two waves of smaller blocks, the second almost empty, 1.26 times)."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    s = W.solvated(W.chain(60))
+    sysh = B.grp_create_system(s, B.GRP_FP64 if prec == "fp64" else B.GRP_MIXED)
+    q0, p0 = W.replica_states(s, 4 * sms, seed=3, spread=0.002)
+    ms = []
+    for R in (2 * sms, 4 * sms):
+        rep = B.grp_init_replicas(sysh, R, SEED, q0[:R], p0[:R], per_replica=True)
+        ms.append(_best_ms(lambda: B.grp_step_k(rep, 10, 10)))
+    assert ms[1] <= 1.15 * 2.0 * ms[0]
