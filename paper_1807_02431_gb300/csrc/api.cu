@@ -1089,7 +1089,12 @@ extern "C" grp_status grp_batch_create(grp_replicas *const *runs, int32_t n_runs
   b->threads = std::min(512, b->threads);
   bool items = true;
   for (int i = 0; i < n_runs; ++i) items = items && !runs[i]->sys->dev.tiled;
-  if (items) b->threads = batch_threads(b->precision, b->threads, b->smem, (int)units.size());
+  if (items) {
+    std::vector<UnitGroup> groups;
+    for (int i = 0; i < n_runs; ++i) groups.push_back(UnitGroup{runs[i]->sys->dev.n_items, runs[i]->R});
+    std::stable_sort(groups.begin(), groups.end(), [](const UnitGroup &x, const UnitGroup &y) { return x.items > y.items; });
+    b->threads = batch_threads(batch_config(b->precision, b->threads, b->smem), groups.data(), n_runs);
+  }
   b->n_units = (int)units.size();
   b->n_branch_units = (int)bunits.size();
   b->n_gr_units = (int)gunits.size();

@@ -60,8 +60,13 @@ struct SegConfig {
 constexpr size_t kMaxSmem = 227 * 1024;
 
 SegConfig segment_config(const SysDev &S, int threads_hint);
-// Block size of the batched kernel for `units` replicas of item-table systems that take up to `threads` each.
-int batch_threads(int precision, int threads, size_t smem, int units);
+// Block sizes of the batched kernel for item-table systems that take up to `threads` each (n_choices, choice, slots,
+// sms), and the one for `count` replicas of each of n groups of systems of `items` items, largest first.
+struct UnitGroup {
+  int items, count;
+};
+SegConfig batch_config(int precision, int threads, size_t smem);
+int batch_threads(const SegConfig &c, const UnitGroup *g, int n);
 // The noise amplitude of every atom in FP64 and FP32 (the system's tables for lean replica states).
 cudaError_t launch_noise_sd(const SysDev &S, double c1, double *sd_d, float *sd_f, cudaStream_t st);
 cudaError_t launch_segment(const SegArgs &a, const SegConfig &cfg, cudaStream_t st);

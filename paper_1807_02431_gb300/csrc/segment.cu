@@ -998,16 +998,53 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
   return c;
 }
 
-int batch_threads(int precision, int threads, size_t smem, int units) {
-  int cand[kMaxThreadChoices], sms = 0;
-  const int n = thread_candidates(threads, cand);
-  for (int t = 0; t < n; ++t) {
-    const int slots = precision == GRP_FP64 ? resident_blocks(ff_segment_batch_kernel<PathF64>, cand[t], smem, sms)
-                                            : resident_blocks(ff_segment_batch_kernel<PathMixed>, cand[t], smem, sms);
-    if (slots == 0) return threads;
-    if (units <= slots) return cand[t];
+SegConfig batch_config(int precision, int threads, size_t smem) {
+  SegConfig c{};
+  c.n_choices = thread_candidates(threads, c.choice);
+  for (int t = 0; t < c.n_choices; ++t) {
+    c.slots[t] = precision == GRP_FP64 ? resident_blocks(ff_segment_batch_kernel<PathF64>, c.choice[t], smem, c.sms)
+                                       : resident_blocks(ff_segment_batch_kernel<PathMixed>, c.choice[t], smem, c.sms);
+    if (c.slots[t] == 0) c.n_choices = 1;
   }
-  return cand[n - 1];
+  return c;
+}
+
+// A batch's blocks take units from a queue, the largest first, so its time is not in waves: at least the work shared out
+// over the places, and k times the k-th unit that one of the places gets, in units of the largest replica's time (800 +
+// items, from replicas of 128 to 1,856 items alone on their SMs).  p blocks per SM slow each other by p^e as in
+// single runs.  us per 40 steps (mixed), 512 threads everywhere -> a size by the number of units alone -> now: 32 replicas of
+// 60 beads and 224 of 10, 199 -> 342 -> 201; 64 each of 10, 22, 40, 60 beads 210 -> 342 -> 212; 128 of 10 and 128 of 60
+// 259 -> 341 -> 261; twice as many 441 -> 476 -> 375; 256 of 60 beads 384 -> 346 -> 343; FP64, 32 of 60 and 224 of 10, 1,234 ->
+// 2,165 -> 1,240.
+int batch_threads(const SegConfig &c, const UnitGroup *g, int n) {
+  long long units = 0;
+  double work = 0.0;
+  const double whole = n > 0 ? 800.0 + g[0].items : 1.0;
+  for (int i = 0; i < n; ++i) {
+    units += g[i].count;
+    work += g[i].count * (800.0 + g[i].items) / whole;
+  }
+  if (c.n_choices < 2 || units == 0) return c.choice[0];
+  const double e = crowding_of(g[0].items, false);
+  int best = 0;
+  double least = 1e300;
+  for (int t = 0; t < c.n_choices; ++t) {
+    const int slots = c.slots[t];
+    double time = work / slots;
+    long long before = 0, k = 0;  // units of larger systems; places filled k times
+    for (int i = 0; i < n; ++i) {
+      const double unit = (800.0 + g[i].items) / whole;
+      before += g[i].count;
+      for (; k * slots < before; ++k) time = std::max(time, (k + 1) * unit);
+    }
+    const long long per_sm = std::min((long long)slots / c.sms, (units + c.sms - 1) / c.sms);
+    const double cost = time * std::pow((double)per_sm, e);
+    if (cost < least * (1.0 - 1e-9)) {
+      least = cost;
+      best = t;
+    }
+  }
+  return c.choice[best];
 }
 
 template <class P>

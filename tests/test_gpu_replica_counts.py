@@ -163,3 +163,20 @@ def test_twice_the_replicas_take_twice_as_long(B, prec):
         rep = B.grp_init_replicas(sysh, R, SEED, q0[:R], p0[:R], per_replica=True)
         ms.append(_best_ms(lambda: B.grp_step_k(rep, 10, 10)))
     assert ms[1] <= 1.15 * 2.0 * ms[0]
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("sizes", [(60, 10, 10, 10, 10, 10, 10, 10), (10, 22, 40, 60)])
+def test_uneven_batches_keep_large_blocks(B, sizes, prec):
+    """A few large replicas among many small ones decide a batch's time: 256 units of uneven sizes take at most 1.25 times
+    as long as a batch of the largest runs alone (with blocks for 256 even units they took 1.6 times)."""
+    p = B.GRP_FP64 if prec == "fp64" else B.GRP_MIXED
+    runs = []
+    for i in range(8):
+        s = W.chain(sizes[i % len(sizes)])
+        q0, p0 = W.replica_states(s, 32, seed=i, spread=0.002)
+        runs.append(B.grp_init_replicas(B.grp_create_system(s, p), 32, SEED + i, q0, p0, per_replica=True))
+    largest = [r for i, r in enumerate(runs) if sizes[i % len(sizes)] == 60]
+    k = 40 if prec == "mixed" else 10
+    ms = [_best_ms(lambda b=B.grp_batch_create(x): B.grp_batch_step_k(b, k, 10)) for x in (largest, runs)]
+    assert ms[1] <= 1.25 * ms[0]
