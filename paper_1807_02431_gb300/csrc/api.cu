@@ -1037,7 +1037,11 @@ extern "C" grp_status grp_gelman_rubin(grp_replicas *r, double tol, double *h_rh
 struct grp_batch {
   std::vector<grp_replicas *> runs;
   int precision = 0;
-  int threads = 0;
+  int threads = 0;             // of every segment, where there is no choice
+  int tuned = 0;               // of every segment, once tuned
+  SegConfig cfg{};             // block sizes that segments choose from (item-table systems)
+  std::vector<int> by_items;   // the runs, those of the largest systems first
+  std::vector<UnitGroup> groups;  // scratch of the choice
   size_t smem = 0;
   int n_units = 0, n_branch_units = 0, n_gr_units = 0;
   SegArgs *d_args = nullptr, *h_args = nullptr;      // [n_runs], h_ pinned
@@ -1089,12 +1093,10 @@ extern "C" grp_status grp_batch_create(grp_replicas *const *runs, int32_t n_runs
   b->threads = std::min(512, b->threads);
   bool items = true;
   for (int i = 0; i < n_runs; ++i) items = items && !runs[i]->sys->dev.tiled;
-  if (items) {
-    std::vector<UnitGroup> groups;
-    for (int i = 0; i < n_runs; ++i) groups.push_back(UnitGroup{runs[i]->sys->dev.n_items, runs[i]->R});
-    std::stable_sort(groups.begin(), groups.end(), [](const UnitGroup &x, const UnitGroup &y) { return x.items > y.items; });
-    b->threads = batch_threads(batch_config(b->precision, b->threads, b->smem), groups.data(), n_runs);
-  }
+  if (items) b->cfg = batch_config(b->precision, b->threads, b->smem);
+  for (int i = 0; i < n_runs; ++i) b->by_items.push_back(i);
+  std::stable_sort(b->by_items.begin(), b->by_items.end(),
+                   [&](int x, int y) { return runs[x]->sys->dev.n_items > runs[y]->sys->dev.n_items; });
   b->n_units = (int)units.size();
   b->n_branch_units = (int)bunits.size();
   b->n_gr_units = (int)gunits.size();
@@ -1151,10 +1153,21 @@ static void fill_args(grp_batch *b, int k, const RunTick *ticks) {
   }
 }
 
-static grp_status enqueue_segment(grp_batch *b, cudaStream_t st) {
+// The block size of a segment, by the replicas that advance in it: the blocks that suit every replica of every run are
+// too small where most runs are in a transient and advance one (64 runs of 32 alkanes, all in transients, 50 ticks of 100
+// steps: 20.7 ms with the 32 threads of 2,048 replicas, 13.2 with the 128 of 64).
+static int segment_threads(grp_batch *b, const RunTick *ticks) {
+  if (b->tuned) return b->tuned;
+  if (b->cfg.n_choices < 2) return b->threads;
+  b->groups.clear();
+  for (int i : b->by_items)
+    if (ticks[i].n_active > 0) b->groups.push_back(UnitGroup{b->runs[i]->sys->dev.n_items, ticks[i].n_active});
+  return batch_threads(b->cfg, b->groups.data(), (int)b->groups.size());
+}
+
+static grp_status enqueue_segment(grp_batch *b, int threads, cudaStream_t st) {
   CU(cudaMemcpyAsync(b->d_args, b->h_args, sizeof(SegArgs) * b->runs.size(), cudaMemcpyHostToDevice, st));
-  CU(launch_segment_batch(b->d_args, b->d_units, b->n_units, b->d_counter, b->precision, b->threads, b->smem, st,
-                          nullptr));
+  CU(launch_segment_batch(b->d_args, b->d_units, b->n_units, b->d_counter, b->precision, threads, b->smem, st, nullptr));
   return GRP_OK;
 }
 
@@ -1162,7 +1175,7 @@ static grp_status enqueue_segment(grp_batch *b, cudaStream_t st) {
 static grp_status batch_launch(grp_batch *b, int k, const RunTick *ticks, cudaStream_t st) {
   CU(cudaStreamSynchronize(st));  // the pinned argument block may still be read by a queued copy
   fill_args(b, k, ticks);
-  return enqueue_segment(b, st);
+  return enqueue_segment(b, segment_threads(b, ticks), st);
 }
 
 // Every replica of every run, with or without the fused exit test.
@@ -1213,8 +1226,8 @@ static grp_status batch_status(grp_batch *b, const int *branch, const int *gr, c
 }
 
 // One tick of the batched loop as a CUDA graph: the segment, branching, Gelman-Rubin ratios and the
-// status readback, captured once per grp_batch_run call.  Every node reads fixed buffers (the pinned
-// argument blocks are refilled before each launch), so the graph is replayed as captured.
+// status readback, captured once per grp_batch_run call and block size of the segment.  Every node reads fixed buffers (the
+// pinned argument blocks are refilled before each launch), so the graph is replayed as captured.
 struct TickGraph {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -1223,11 +1236,11 @@ struct TickGraph {
     if (graph) cudaGraphDestroy(graph);
   }
   // false (and no graph) when capture is unavailable; the caller then launches the nodes one by one
-  bool capture(grp_batch *b) {
+  bool capture(grp_batch *b, int threads) {
     cudaStream_t cs = nullptr;
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); return false; }
     bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    const bool queued = ok && enqueue_segment(b, cs) == GRP_OK && enqueue_status(b, cs) == GRP_OK;
+    const bool queued = ok && enqueue_segment(b, threads, cs) == GRP_OK && enqueue_status(b, cs) == GRP_OK;
     if (ok) ok = cudaStreamEndCapture(cs, &graph) == cudaSuccess && queued;
     if (ok) ok = cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
     cudaStreamDestroy(cs);
@@ -1335,7 +1348,7 @@ extern "C" grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *strea
   float best_ms = 1e30f;
   grp_status status = GRP_OK;
   for (int c : candidates) {
-    b->threads = c;
+    b->tuned = c;
     if (batch_segment(b, 10, t_gr, 0, nullptr, st) != GRP_OK) continue;  // warm-up
     cudaEventRecord(e0, st);
     status = batch_segment(b, 50, t_gr, 0, nullptr, st);
@@ -1346,7 +1359,7 @@ extern "C" grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *strea
     cudaEventElapsedTime(&ms, e0, e1);
     if (ms < best_ms) { best_ms = ms; best = c; }
   }
-  b->threads = best;
+  b->tuned = best;
   for (size_t i = 0; i < b->runs.size(); ++i) {
     grp_replicas *r = b->runs[i];
     Snap &s = snaps[i];
@@ -1767,7 +1780,7 @@ extern "C" grp_status grp_batch_run(grp_batch *b, const grp_run_params *p, grp_e
 
   std::vector<RunTick> ticks(nr);
   std::vector<int> branch(nr), gr(nr);
-  TickGraph tick;
+  TickGraph tick[512 / 32];  // by the warps of the segment's blocks
   bool graphs = true;
   long long n_ticks = 0;
   b->ticks = b->graph_ticks = 0;
@@ -1793,16 +1806,18 @@ extern "C" grp_status grp_batch_run(grp_batch *b, const grp_run_params *p, grp_e
       busy += t.n_active > 0;
     }
     if (!busy) break;
-    // the first tick runs node by node (it also sets the kernels' attributes); the graph is captured
-    // before the second and replayed from then on
-    if (graphs && n_ticks == 1 && !tick.capture(b)) graphs = false;
+    // the first tick runs node by node (it also sets the kernels' attributes); from the second on, the graph of a
+    // block size is captured before its first tick and replayed from then on
+    const int threads = segment_threads(b, ticks.data());
+    TickGraph &g = tick[threads / 32 - 1];
+    if (graphs && n_ticks > 0 && !g.exec && !g.capture(b, threads)) graphs = false;
     fill_args(b, p->t_check, ticks.data());
     fill_arrays(b, branch.data(), gr.data());
-    if (graphs && tick.exec) {
-      CU(cudaGraphLaunch(tick.exec, st));
+    if (graphs && g.exec) {
+      CU(cudaGraphLaunch(g.exec, st));
       ++b->graph_ticks;
     } else {
-      if ((e = enqueue_segment(b, st)) != GRP_OK) return e;
+      if ((e = enqueue_segment(b, threads, st)) != GRP_OK) return e;
       if ((e = enqueue_status(b, st)) != GRP_OK) return e;
     }
     CU(cudaStreamSynchronize(st));

@@ -180,3 +180,23 @@ def test_uneven_batches_keep_large_blocks(B, sizes, prec):
     k = 40 if prec == "mixed" else 10
     ms = [_best_ms(lambda b=B.grp_batch_create(x): B.grp_batch_step_k(b, k, 10)) for x in (largest, runs)]
     assert ms[1] <= 1.25 * ms[0]
+
+
+def test_transients_of_a_batch_keep_large_blocks(B):
+    """Runs in a transient advance one replica each, whatever their sets: 64 runs of 32 replicas take at most 1.25 times as
+    long as 64 of 4 (with the blocks of 2,048 replicas they took 1.6 times), and see the same events."""
+    s = W.alkane(core_half_width=0.01)  # hardly ever inside a state's core
+    out = []
+    for R in (4, 32):
+        sysh = B.grp_create_system(s, B.GRP_MIXED)
+        runs = []
+        for i in range(64):
+            q0, p0 = W.replica_states(s, R, seed=i, spread=0.002)
+            q0[:], p0[:] = W.replica_states(s, 1, seed=i, spread=0.02)[0], W.replica_states(s, 1, seed=i)[1]
+            runs.append(B.grp_init_replicas(sysh, R, SEED + i, q0, p0, per_replica=True))
+        batch, ends = B.grp_batch_create(runs), iter(range(2000, 20000, 2000))
+        out.append((_best_ms(lambda: B.grp_batch_run(batch, 10, 100, 0.05, 1000, next(ends), 100), 4),
+                    [B.grp_get_state(r)[0][0] for r in runs]))
+    assert out[1][0] <= 1.25 * out[0][0]
+    for a, b in zip(out[0][1], out[1][1]):
+        assert np.array_equal(a, b)
