@@ -372,7 +372,8 @@ grp_status grp_batch_run(grp_batch *b, const grp_run_params *p, grp_event *h_eve
  * but the first, unless the capture was unavailable and every tick was launched node by node). */
 grp_status grp_batch_stats(const grp_batch *b, int64_t *h_ticks, int64_t *h_graph_ticks);
 /* Pick the block size of the batched kernel by timing candidate sizes on a short segment (the
- * replicas' state and counters are restored afterwards); h_threads (optional) gets the choice. */
+ * replicas' state and counters are restored afterwards); the size in use stays unless another is faster.
+ * h_threads (optional) gets the size of segments of every replica. */
 grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *stream, int32_t *h_threads);
 
 /* Whole loop of Fig. 1 from the current state of replica 0: transient, convergence (F-V with

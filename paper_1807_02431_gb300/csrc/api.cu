@@ -1038,7 +1038,7 @@ struct grp_batch {
   std::vector<grp_replicas *> runs;
   int precision = 0;
   int threads = 0;             // of every segment, where there is no choice
-  int tuned = 0;               // of every segment, once tuned
+  int tuned = 0;               // of every segment, where tuning found a faster one
   SegConfig cfg{};             // block sizes that segments choose from (item-table systems)
   std::vector<int> by_items;   // the runs, those of the largest systems first
   std::vector<UnitGroup> groups;  // scratch of the choice
@@ -1340,11 +1340,16 @@ extern "C" grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *strea
     s.tp = r->t_phase;
     snaps.push_back(s);
   }
-  const int candidates[] = {128, 256, 384, 512};
+  // first what runs untuned (0), which another has to beat by 2 %: two runs of one size differ by less
+  std::vector<int> candidates = {0, 128, 256, 384, 512};
+  for (int t = 0; t < b->cfg.n_choices; ++t) {
+    const int c = b->cfg.choice[t];
+    if (std::find(candidates.begin(), candidates.end(), c) == candidates.end()) candidates.push_back(c);
+  }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  int best = b->threads;
+  int best = 0;
   float best_ms = 1e30f;
   grp_status status = GRP_OK;
   for (int c : candidates) {
@@ -1357,7 +1362,7 @@ extern "C" grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *strea
     cudaEventSynchronize(e1);
     float ms = 0;
     cudaEventElapsedTime(&ms, e0, e1);
-    if (ms < best_ms) { best_ms = ms; best = c; }
+    if (ms < (c == 0 ? best_ms : 0.98f * best_ms)) { best_ms = ms; best = c; }
   }
   b->tuned = best;
   for (size_t i = 0; i < b->runs.size(); ++i) {
@@ -1374,7 +1379,9 @@ extern "C" grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *strea
   for (Snap &s : snaps) { cudaFree(s.q); cudaFree(s.p); cudaFree(s.f); cudaFree(s.acc); }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (h_threads) *h_threads = best;
+  std::vector<RunTick> all(b->runs.size());
+  for (size_t i = 0; i < all.size(); ++i) all[i].n_active = b->runs[i]->R;
+  if (h_threads) *h_threads = segment_threads(b, all.data());
   return status;
 }
 

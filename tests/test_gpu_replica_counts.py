@@ -200,3 +200,20 @@ def test_transients_of_a_batch_keep_large_blocks(B):
     assert out[1][0] <= 1.25 * out[0][0]
     for a, b in zip(out[0][1], out[1][1]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("make,n_runs,R", [("alkane", 64, 32), ("chain22", 8, 40), ("mixed sizes", 8, 32)])
+def test_autotuning_keeps_the_faster_block_size(B, make, n_runs, R):
+    """A batch is no slower after its tuning than before (1.15: two timings of one size differ by less), and tuning it
+    again finds the same; small systems' own sizes are among the candidates."""
+    runs = []
+    for i in range(n_runs):
+        s = W.alkane() if make == "alkane" else W.chain(22 if make == "chain22" else (10, 22, 40, 60)[i % 4])
+        q0, p0 = W.replica_states(s, R, seed=i, spread=0.002)
+        runs.append(B.grp_init_replicas(B.grp_create_system(s, B.GRP_MIXED), R, SEED + i, q0, p0, per_replica=True))
+    batch = B.grp_batch_create(runs)
+    ms = [_best_ms(lambda: B.grp_batch_step_k(batch, 100, 10))]
+    for _ in range(2):
+        assert 32 <= B.grp_batch_autotune(batch, 10) <= 512
+        ms.append(_best_ms(lambda: B.grp_batch_step_k(batch, 100, 10)))
+    assert max(ms[1:]) <= 1.15 * ms[0]
