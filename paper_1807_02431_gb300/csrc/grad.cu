@@ -252,7 +252,7 @@ cudaError_t launch_param_grad(const SysDev &S, int n_terms, int n_conf, const do
   cudaError_t e;
   if (S.precision == GRP_FP64) {
     auto k = param_grad_kernel<double, double4, double4, false>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = allow_smem(k)) != cudaSuccess) return e;
     k<<<n_conf, 256, smem, st>>>(S, S.atom_d, S.term_d, n_terms, q, w, grad_q, partial, err);
   } else {
     // staged while two blocks share an SM
@@ -260,7 +260,7 @@ cudaError_t launch_param_grad(const SysDev &S, int n_terms, int n_conf, const do
     const bool fits = staged <= 113 * 1024;
     auto k = fits ? param_grad_kernel<float, float4, float4, true> : param_grad_kernel<float, float4, float4, false>;
     const size_t bytes = fits ? staged : smem;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if ((e = allow_smem(k)) != cudaSuccess) return e;
     k<<<n_conf, 256, bytes, st>>>(S, S.atom_f, S.term_f, n_terms, q, w, grad_q, partial, err);
   }
   return cudaGetLastError();
@@ -568,7 +568,7 @@ cudaError_t launch_adjoint(const AdjArgs &a, int n_rep, cudaStream_t st) {
   const bool fewer = (n_rep + three - 1) / three < (n_rep + two - 1) / two;
   auto kern = a.S.precision == GRP_FP64 ? adjoint_kernel<PathF64, 2>
                                         : (fewer ? adjoint_kernel<PathMixed, 3> : adjoint_kernel<PathMixed, 2>);
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  if ((e = allow_smem(kern)) != cudaSuccess) return e;
   kern<<<n_rep, 256, smem, st>>>(a);
   return cudaGetLastError();
 }

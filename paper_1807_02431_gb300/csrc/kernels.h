@@ -56,8 +56,17 @@ struct SegConfig {
   double crowding;  // a wave of p blocks per SM takes p^crowding of the time of one block per SM
 };
 
-// Largest dynamic shared memory of one block on sm_103a.
+// Largest shared memory of one block on sm_103a, and the batched kernel's static part of it.
 constexpr size_t kMaxSmem = 227 * 1024;
+constexpr size_t kBatchStaticSmem = 1120;
+
+// Allows a kernel's launches all the dynamic shared memory that its static variables leave.  The limit is the kernel's,
+// in every thread and for every system: set to what each launch or query needs, one thread lowered it between another's
+// setting and its launch, which was then refused.  The same value every time, nothing can be lowered.
+template <class K>
+inline cudaError_t allow_smem(K *kern, size_t static_bytes = 0) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem - static_bytes));
+}
 
 SegConfig segment_config(const SysDev &S, int threads_hint);
 // Block sizes of the batched kernel for item-table systems that take up to `threads` each (n_choices, choice, slots,

@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(512, 1) ff_segment_batch_kernel(const SegArgs 
   __shared__ SegArgs sa;
   __shared__ int su;
   // beside the replica's state, which takes the rest of the 227 KB for systems of 2,380 to 2,500 atoms
-  static_assert(sizeof(SegArgs) + 8 <= 1120, "a larger SegArgs takes the largest systems out of batches");
+  static_assert(sizeof(SegArgs) + 8 <= kBatchStaticSmem, "a larger SegArgs takes the largest systems out of batches");
   for (;;) {
     if (threadIdx.x == 0) {
       // units of replicas beyond a run's n_active (a transient advances replica 0 alone, a finished
@@ -884,9 +884,9 @@ static auto ff_kernel(const SysDev &S, int threads) {
 
 // Blocks of the kernel that the device holds at once (0: unknown).
 template <class K>
-static int resident_blocks(K kern, int threads, size_t smem, int &sms) {
+static int resident_blocks(K kern, int threads, size_t smem, size_t static_smem, int &sms) {
   int dev = 0, per_sm = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (allow_smem(kern, static_smem) != cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess) {
@@ -990,8 +990,8 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
     c.crowding = crowding_of(S.n_items, S.n_cons > 0);
     for (int t = 0; t < c.n_choices; ++t) {
       c.slots[t] = S.precision == GRP_FP64
-                       ? resident_blocks(ff_kernel<PathF64>(S, c.choice[t]), c.choice[t], c.smem, c.sms)
-                       : resident_blocks(ff_kernel<PathMixed>(S, c.choice[t]), c.choice[t], c.smem, c.sms);
+                       ? resident_blocks(ff_kernel<PathF64>(S, c.choice[t]), c.choice[t], c.smem, 0, c.sms)
+                       : resident_blocks(ff_kernel<PathMixed>(S, c.choice[t]), c.choice[t], c.smem, 0, c.sms);
       if (c.slots[t] == 0) c.n_choices = 1;  // nothing known: the default
     }
   }
@@ -1002,8 +1002,9 @@ SegConfig batch_config(int precision, int threads, size_t smem) {
   SegConfig c{};
   c.n_choices = thread_candidates(threads, c.choice);
   for (int t = 0; t < c.n_choices; ++t) {
-    c.slots[t] = precision == GRP_FP64 ? resident_blocks(ff_segment_batch_kernel<PathF64>, c.choice[t], smem, c.sms)
-                                       : resident_blocks(ff_segment_batch_kernel<PathMixed>, c.choice[t], smem, c.sms);
+    c.slots[t] = precision == GRP_FP64
+                     ? resident_blocks(ff_segment_batch_kernel<PathF64>, c.choice[t], smem, kBatchStaticSmem, c.sms)
+                     : resident_blocks(ff_segment_batch_kernel<PathMixed>, c.choice[t], smem, kBatchStaticSmem, c.sms);
     if (c.slots[t] == 0) c.n_choices = 1;
   }
   return c;
@@ -1052,7 +1053,7 @@ static cudaError_t launch_ff_p(const SegArgs &a, const SegConfig &c, cudaStream_
   const int threads = c.n_choices > 1 ? choose_threads(c, a.n_active) : c.threads;
   if (threads < 32 || threads > 512 || threads % 32) return cudaErrorInvalidValue;
   auto kern = ff_kernel<P>(a.S, threads);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);
+  cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   kern<<<a.n_active, threads, c.smem, st>>>(a, c.rows);
   return cudaGetLastError();
@@ -1063,7 +1064,8 @@ cudaError_t launch_segment_batch(const SegArgs *d_runs, const uint2 *d_units, in
   if (n_units <= 0) return cudaSuccess;
   if (threads < 32 || threads > 512 || threads % 32) return cudaErrorInvalidValue;
   auto kern = precision == GRP_FP64 ? ff_segment_batch_kernel<PathF64> : ff_segment_batch_kernel<PathMixed>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > kMaxSmem - kBatchStaticSmem) return cudaErrorInvalidValue;
+  cudaError_t e = allow_smem(kern, kBatchStaticSmem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1214,10 +1216,10 @@ cudaError_t launch_energy_forces(const SysDev &S, int n_conf, const double *q, d
     if (e != cudaSuccess) return e;
   }
   if (S.precision == GRP_FP64) {
-    e = cudaFuncSetAttribute(energy_forces_kernel<PathF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(energy_forces_kernel<PathF64>);
     if (e == cudaSuccess) energy_forces_kernel<PathF64><<<n_conf, 256, smem, st>>>(S, q, energy, forces, err, lean, gb_glob);
   } else {
-    e = cudaFuncSetAttribute(energy_forces_kernel<PathMixed>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(energy_forces_kernel<PathMixed>);
     if (e == cudaSuccess) energy_forces_kernel<PathMixed><<<n_conf, 256, smem, st>>>(S, q, energy, forces, err, lean, gb_glob);
   }
   if (e == cudaSuccess) e = cudaGetLastError();
