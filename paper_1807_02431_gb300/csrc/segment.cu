@@ -724,9 +724,9 @@ __global__ void __launch_bounds__(512, 1) ff_segment_batch_kernel(const SegArgs 
 // operations per coordinate; its normals (a logarithm, a square root and a sine and cosine) do not depend on the
 // state.  So a block of four warps draws the normals of 128 / G steps at a time for its G replicas, one (step,
 // replica) per thread, and its first warp then runs the steps, one lane per coordinate (the two coordinates
-// meet only in the sampled energies).  G = 1 spreads the replicas over the SMs, up to eight chains per SM; more
-// replicas fill the lanes of the stepping warp.  (One thread per replica drawing its normals in the chain: 333 us
-// for 32 replicas x 100 steps; now 50.)
+// meet only in the sampled energies).  G = 1 spreads the replicas over the SMs; more replicas fill the lanes of
+// the stepping warp (launch_dw).  (One thread per replica drawing its normals in the chain: 333 us for 32 replicas x 100
+// steps; now 50.)
 template <int G>
 __global__ void __launch_bounds__(128) dw_segment_kernel(const __grid_constant__ SegArgs a) {
   constexpr int NB = 128 / G;
@@ -811,11 +811,13 @@ __global__ void __launch_bounds__(128) dw_segment_kernel(const __grid_constant__
   }
 }
 
-static cudaError_t launch_dw(const SegArgs &a, cudaStream_t st) {
+// One replica per block up to three per SM, four up to sixteen per SM, then sixteen: where their times cross (152 SMs, 200
+// steps, us with 1 | 4 | 16: 152 replicas 104 | 120 | 174, 456 117 | 120 | 174, 608 129 | 120 | 174, 912 181 | 135 | 174, 1,216
+// 266 | 134 | 175, 2,432 462 | 176 | 176, 3,648 696 | 254 | 234, 4,864 937 | 365 | 234, 65,536 11,955 | 4,288 | 2,495).
+static cudaError_t launch_dw(const SegArgs &a, const SegConfig &c, cudaStream_t st) {
   const int R = a.n_active;
-  // up to eight blocks per SM of a 152-SM part with one replica each, then with four; more in full warps
-  if (R <= 1216) dw_segment_kernel<1><<<R, 128, 0, st>>>(a);
-  else if (R <= 4864) dw_segment_kernel<4><<<(R + 3) / 4, 128, 0, st>>>(a);
+  if (R <= 3 * c.sms) dw_segment_kernel<1><<<R, 128, 0, st>>>(a);
+  else if (R <= 16 * c.sms) dw_segment_kernel<4><<<(R + 3) / 4, 128, 0, st>>>(a);
   else dw_segment_kernel<16><<<(R + 15) / 16, 128, 0, st>>>(a);
   return cudaGetLastError();
 }
@@ -947,6 +949,12 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
     c.threads = 64;
     c.smem = 0;
     c.noise_batch = 1;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      c.sms = 0;  // unknown: sixteen replicas per block
+    }
     return c;
   }
   // one thread per (padded) item, or one warp per tile pair, up to 512 threads per replica, a
@@ -1087,7 +1095,7 @@ cudaError_t launch_segment(const SegArgs &a0, const SegConfig &c, cudaStream_t s
   a.lean = c.lean;
   if (a.n_active <= 0) return cudaSuccess;
   if (a.S.potential == GRP_POT_DOUBLE_WELL_2D) {
-    return launch_dw(a, st);
+    return launch_dw(a, c, st);
   }
   return a.S.precision == GRP_FP64 ? launch_ff_p<PathF64>(a, c, st) : launch_ff_p<PathMixed>(a, c, st);
 }

@@ -217,3 +217,35 @@ def test_autotuning_keeps_the_faster_block_size(B, make, n_runs, R):
         assert 32 <= B.grp_batch_autotune(batch, 10) <= 512
         ms.append(_best_ms(lambda: B.grp_batch_step_k(batch, 100, 10)))
     assert max(ms[1:]) <= 1.15 * ms[0]
+
+
+@pytest.mark.parametrize("per_sm", [(3, 8), (4, 8), (6, 9), (16, 32), (20, 32)])
+def test_double_well_time_grows_with_replicas(B, per_sm):
+    """A smaller set is no slower than a larger one (1.1: two timings of one differ by less): the number of replicas per
+    block changes where the times cross.  (With one per block up to eight per SM, 913 to 1,216 replicas took 1.7 times as
+    long as 1,217, and up to 32 per SM with four, 3,649 to 4,864 took 1.2 times as long as 4,865.)"""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ms = []
+    for R in (per_sm[0] * sms, per_sm[0] * sms + 1, per_sm[1] * sms, per_sm[1] * sms + 1):
+        s = W.double_well_2d(n_replicas=R)
+        q0, p0 = W.replica_states(s, R, seed=3, spread=0.1)
+        rep = B.grp_init_replicas(B.grp_create_system(s, B.GRP_FP64), R, SEED, q0, p0, per_replica=True)
+        ms.append(_best_ms(lambda: B.grp_step_k(rep, 2000, 10)))
+    assert all(a <= 1.1 * b for a, b in zip(ms, ms[1:]))
+
+
+@pytest.mark.parametrize("R", [456, 457, 459, 2432, 2433, 2447])
+def test_double_well_lines(B, R):
+    """On both sides of the lines: the last replicas are those of the shard that starts there, in a small set."""
+    s = W.double_well_2d(n_replicas=R)
+    q0, p0 = W.replica_states(s, R, seed=3, spread=0.2)
+    sysh = B.grp_create_system(s, B.GRP_FP64)
+    rep = B.grp_init_replicas(sysh, R, SEED, q0, p0, per_replica=True)
+    B.grp_step_k(rep, 130, 5)
+    part = B.grp_init_replicas(sysh, 7, SEED, q0[R - 7:], p0[R - 7:], per_replica=True)
+    B.grp_set_shard(part, R - 7, R)
+    B.grp_step_k(part, 130, 5)
+    for a, b in zip(B.grp_get_state(rep)[:3], B.grp_get_state(part)[:3]):
+        assert np.array_equal(a[R - 7:], b)
