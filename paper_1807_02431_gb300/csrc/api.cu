@@ -494,13 +494,22 @@ extern "C" grp_status grp_create_system(const grp_system_desc *d, grp_system **o
       rows.n_stiff = (int)stiff.size();
       UP(stiff.data(), stiff.size(), &rows.stiff);
       // a pair is on the row of its lower atom when the sum of the two is odd, of the higher when it is even, so
-      // that every atom has about half of its neighbours on its row
+      // that every atom has about half of its neighbours on its row: whole words by tile, less the excluded pairs
       const int nt = D.n_tiles;
       std::vector<uint32_t> rmask((size_t)nt * nt * 32, 0);
-      for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j)
-          if (i != j && !excl[(size_t)i * n + j] && (((i + j) & 1) ? i < j : i > j))
-            rmask[((size_t)(i / 32) * nt + j / 32) * 32 + i % 32] |= 1u << (j % 32);
+      auto word = [&](int i, int J) -> uint32_t & { return rmask[((size_t)(i / 32) * nt + J) * 32 + i % 32]; };
+      for (int i = 0; i < n; ++i) {
+        const int l = i % 32;
+        const uint32_t odd = (l & 1) ? 0x55555555u : 0xAAAAAAAAu, above = l == 31 ? 0u : ~0u << (l + 1), below = (1u << l) - 1u;
+        for (int J = 0; J < nt; ++J)
+          word(i, J) = J > i / 32 ? odd : (J < i / 32 ? ~odd : (odd & above) | (~odd & below));
+        if (n % 32) word(i, nt - 1) &= (1u << (n % 32)) - 1u;
+      }
+      for (int e = 0; e < d->n_excl; ++e) {
+        const int i = d->excl[2 * e], j = d->excl[2 * e + 1];
+        word(i, j / 32) &= ~(1u << (j % 32));
+        word(j, i / 32) &= ~(1u << (i % 32));
+      }
       UP(rmask.data(), rmask.size(), &rows.masks);
     }
     D.n_bonds = d->n_bonds;

@@ -171,3 +171,20 @@ def test_rows_outgrown_by_one_replica(B, hub):
         B.grp_batch_step_k(B.grp_batch_create([run]), k, 10)
         for a, b in zip(B.grp_get_state(alone)[:3], B.grp_get_state(run)[:3]):
             assert np.array_equal(a, b)
+
+
+def test_systems_with_rows_are_made_quickly(B):
+    """The rows' tables add at most a third to the time in which a system is made: one of 1,024 atoms against one of 1,022,
+    which has none (they more than doubled it)."""
+    import time
+
+    def best(n):
+        s = _gas(n, 1.2)
+        t = []
+        for _ in range(7):
+            t0 = time.perf_counter()
+            B.grp_create_system(s, B.GRP_MIXED)
+            t.append(time.perf_counter() - t0)
+        return min(t)
+
+    assert best(1024) <= 1.33 * best(1022)
