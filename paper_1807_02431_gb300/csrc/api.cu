@@ -1350,11 +1350,16 @@ extern "C" grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *strea
     snaps.push_back(s);
   }
   // first what runs untuned (0), which another has to beat by 2 %: two runs of one size differ by less
-  std::vector<int> candidates = {0, 128, 256, 384, 512};
-  for (int t = 0; t < b->cfg.n_choices; ++t) {
-    const int c = b->cfg.choice[t];
-    if (std::find(candidates.begin(), candidates.end(), c) == candidates.end()) candidates.push_back(c);
-  }
+  std::vector<RunTick> all(b->runs.size());
+  for (size_t i = 0; i < all.size(); ++i) all[i].n_active = b->runs[i]->R;
+  b->tuned = 0;
+  const int untuned = segment_threads(b, all.data());
+  std::vector<int> candidates = {0};
+  auto add = [&](int c) {
+    if (c != untuned && std::find(candidates.begin(), candidates.end(), c) == candidates.end()) candidates.push_back(c);
+  };
+  for (int c : {128, 256, 384, 512}) add(c);
+  for (int t = 0; t < b->cfg.n_choices; ++t) add(b->cfg.choice[t]);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -1388,9 +1393,7 @@ extern "C" grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *strea
   for (Snap &s : snaps) { cudaFree(s.q); cudaFree(s.p); cudaFree(s.f); cudaFree(s.acc); }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  std::vector<RunTick> all(b->runs.size());
-  for (size_t i = 0; i < all.size(); ++i) all[i].n_active = b->runs[i]->R;
-  if (h_threads) *h_threads = segment_threads(b, all.data());
+  if (h_threads) *h_threads = best ? best : untuned;
   return status;
 }
 
