@@ -28,8 +28,9 @@ constexpr double kFixLimit = 4194304.0;               // 2^22
 // Mixed path: bonds at least this stiff (kJ/mol/nm^2) take r - r0 in double-single arithmetic.
 constexpr float kSoftBond = 1.0e4f;
 // Systems in vacuum on the mixed path keep neighbour rows from this size on: two tiles for each of a block's sixteen
-// warps (1,024 atoms, 40 replicas x 60 steps, 3.7 -> 2.9 ms; 2,030 atoms 11.5 -> 9.6 with 200).  With seven tiles (220
-// atoms in a periodic box) rows were slower than the pair list.
+// warps.  Pairs -> rows, 152 replicas x 60 steps, ligand models: 1,000 atoms 3.27 -> 2.63 ms, 768 2.56 -> 2.17, 512 1.54 ->
+// 1.31, 256 0.76 -> 0.79, 128 0.42 -> 0.62: the two cross between 256 and 512 atoms, and from there to the line the pair
+// list still runs.  With seven tiles (220 atoms in a periodic box) rows were slower.
 constexpr int kRowsMinAtoms = 1024;
 // Partners that a row holds.  A replica set whose first configuration has longer rows keeps the pair list (globules of
 // 1,024 atoms with a cutoff of 1.2 nm: from about 50 atoms per nm^3 on).
@@ -211,8 +212,8 @@ __device__ __forceinline__ void normals4_f32(const Philox4 &w, float xi[4]) {
 // The conversion runs on the integer pipe: the significand of v 2^40 shifted to its place and rounded to
 // nearest even, the value of __double2ll_rn(v 2^40) for every |v| < 2^22.  As a compare, a multiply and a
 // conversion it took three instructions of the FP64 pipe, whose rate on sm_103a is 1/64 of the FP32 rate and
-// which bounds the FP64 kernels (22 beads, 256 replicas x 500 steps: 8.09 -> 7.07 ms, 7.29 with the dihedrals out of line; parameter gradient of 2,048
-// configurations of 100 beads, mixed: 535 -> 245 us).
+// which bounds the FP64 kernels (22 beads, 256 replicas x 500 steps: 8.09 -> 7.07 ms, 7.29 with the dihedrals out of line;
+// parameter gradient of 2,048 configurations of 100 beads, mixed: 535 -> 245 us).
 __device__ __forceinline__ long long fix_shift(unsigned long long m, int sh, bool neg) {
   // m 2^sh rounded to an integer, sh <= 9 (double) or <= 38 (float); below 2^-54 every m < 2^53 rounds to 0
   unsigned long long r;

@@ -501,10 +501,11 @@ __device__ __forceinline__ void dihedral_term(const Pos<P> &pos, const Params<P>
 }
 
 // Nonbonded pairs of a Verlet list (i | j << 16), strided over the block's threads; pairs beyond the
-// cutoff contribute nothing; in a periodic box (Ewald real space) each pair takes its nearest image.  The list lives in global memory (L2): each thread loads its next four
-// entries before evaluating them, so that one load latency covers four pairs.  (Measured on the
-// 2,030-atom ligand workload, this pair list with fixed-point atomics on both atoms beat per-atom
-// neighbour rows evaluated from both ends by 1.36x, and rows holding each pair once by 7x.)
+// cutoff contribute nothing; in a periodic box (Ewald real space) each pair takes its nearest image.  The list lives in
+// global memory (L2): each thread loads its next four entries before evaluating them, so that one load latency covers
+// four pairs.  (On the 2,030-atom ligand, pairs with fixed-point atomics on both atoms beat per-atom rows evaluated from
+// both ends by 1.36x; rows that hold each pair once, four partners at a time, beat the pairs by 1.34x, and large systems
+// in vacuum on the mixed path take them: rows.cuh.)
 template <class P, int kRF = -1>
 __device__ __forceinline__ void list_pass(const SysDev &S, const Pos<P> &pos, const Params<P> &par,
                                           const uint32_t *list, int count, const typename P::Acc &acc,

@@ -78,8 +78,8 @@ __device__ __forceinline__ auto gb_atom(const SysDev &S, int i) {
 // by every thread of the block, with the positions final; returns after the last pass (the caller's
 // barrier before reading the forces covers it).  The scratch accumulators are zero on entry and left
 // zero.  A step of such a small system is a chain of latencies, so
-//  * each thread's first pair (the only one up to 25 beads on 320 threads) keeps its difference, distance, charges and
-//    derivatives in registers through the three pair passes;
+//  * each thread's first pair (the only one up to 25 beads on 320 threads, up to 20 on the 192 of larger sets) keeps its
+//    difference, distance, charges and derivatives in registers through the three pair passes;
 //  * `other()`, the vacuum forces, runs beside pass 2, whose one warp of atoms with divisions and a hyperbolic
 //    tangent would keep the rest of the block waiting.
 // 22 beads, 256 replicas x 500 steps: 2.10 -> 1.94 ms.

@@ -909,7 +909,9 @@ static int resident_blocks(K kern, int threads, size_t smem, size_t static_smem,
 // threads), 1,024 replicas 1,614 -> 1,185 (160); 60 beads 256 replicas 855 -> 756; 22 beads 400 replicas 303 -> 231
 // (192), 1,024 replicas 625 -> 485 (160); 24 atoms with constraints, 512 replicas 1,458 -> 856; solvated 22 beads,
 // 512 replicas 826 -> 709; FP64 22 beads, 1,024 replicas 6,470 -> 5,220; batch of 2,048 alkanes of 7 beads 1,277 ->
-// 989 (32).  Sizes between (96, 128, 224, 256) were within 5 % or slower.  The particle mesh keeps its 320.
+// 989 (32).  Not among them: 128 and 96 threads, which suit some counts that fill their waves better (22 beads, 640
+// replicas x 30 steps, 119 us with 128, 140 with 192).  A block has at least 32 threads, one for each of the 4 x 8 words
+// of the sampled observables.  The particle mesh keeps its 320.
 static int thread_candidates(int threads, int out[kMaxThreadChoices]) {
   static const int kLarge[] = {320, 192, 160}, kSmall[] = {64, 32};
   int n = 0;
@@ -923,8 +925,8 @@ static int thread_candidates(int threads, int out[kMaxThreadChoices]) {
   }
   return n;
 }
-// The exponent e: a system of 288 items (22 beads) takes 1.3 times as long with two blocks per SM as with one, of 1,856
-// (60 beads) 1.7 times; with constraints, one warp's chain is the step whatever runs beside it.
+// The exponent e: a step of 288 items (22 beads) takes about 1.3 times as long with two blocks per SM as with one, of
+// 1,856 (60 beads) 1.7 times; with constraints, one warp's chain is the step whatever runs beside it.
 static double crowding_of(int n_items, bool constraints) {
   return constraints ? 0.0 : std::min(0.8, std::sqrt((double)n_items) / 55.0);
 }
@@ -958,7 +960,7 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
     return c;
   }
   // one thread per (padded) item, or one warp per tile pair, up to 512 threads per replica, a
-  // multiple of 32, at least 64
+  // multiple of 32, at least 64 (the default: larger sets of small systems take fewer, thread_candidates)
   int t = threads_hint;
   if (t <= 0) {
     t = ((S.n_items + 31) / 32) * 32;
@@ -967,8 +969,10 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
   t = t < 64 ? 64 : (t > 512 ? 512 : ((t + 31) / 32) * 32);
   // the mixed path's particle mesh and constraints: 320 threads, two replicas per SM (the mesh's 256
   // lines per transform pass take one round of the block; the constraint groups run on one warp, and
-  // two blocks per SM run two such warps at once and 256 replicas in one wave); the FP64 transforms and
-  // groups need the registers of the 512-thread variant
+  // two blocks per SM run two such warps at once and 256 replicas in one wave); the FP64 transforms
+  // need the registers of the 512-thread variant, and FP64 groups start from it: sets that fit take its blocks, larger
+  // ones the candidates' (22 beads with hydrogens, FP64, 30 steps, us by threads: 16 replicas 1,133 with 512; 256 replicas
+  // 2,383 with 512, 1,525 with 320; 1,024 replicas 8,243 with 512, 4,310 with 160)
   if ((S.coulomb_rf == 2 || S.n_cons > 0) && S.precision != GRP_FP64 && threads_hint <= 0 && t > 320 && !S.tiled)
     t = 320;
   c.threads = t;
