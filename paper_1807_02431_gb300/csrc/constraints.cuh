@@ -5,9 +5,7 @@
 // integrates a whole group in FP64 (the mixed path's single-bond groups in double-single, below), with
 // Gauss-Seidel sweeps over the group's
 // constraints in their order until a sweep moves nothing beyond the tolerance, so that the result is
-// that of sweeping over every constraint of the system.  The FP64 arithmetic is written with explicitly rounded
-// operations (as State::baoa_c): a set of other size runs another instantiation of the kernel, and where the compiler
-// chose the contractions, those for blocks of 320 and of 512 threads differed in the last bit.
+// that of sweeping over every constraint of the system.  Item-table systems only.
 #pragma once
 #include "state.cuh"
 
@@ -90,14 +88,14 @@ __device__ bool con_rattle(const SysDev &S, ConGroup &G) {
       const double r[3] = {G.q[i][0] - G.q[j][0], G.q[i][1] - G.q[j][1], G.q[i][2] - G.q[j][2]};
       double rv = 0.0, rr = 0.0;
       for (int x = 0; x < 3; ++x) {
-        rv = __fma_rn(r[x], __fma_rn(G.p[i][x], wi, -__dmul_rn(G.p[j][x], wj)), rv);
-        rr = __fma_rn(r[x], r[x], rr);
+        rv += r[x] * (G.p[i][x] * wi - G.p[j][x] * wj);
+        rr += r[x] * r[x];
       }
       if (fabs(rv) <= S.con_tol * d * d / S.dt) continue;
-      const double mu = rv / __dmul_rn(__dadd_rn(wi, wj), rr);
+      const double mu = rv / ((wi + wj) * rr);
       for (int x = 0; x < 3; ++x) {
-        G.p[i][x] = __fma_rn(-mu, r[x], G.p[i][x]);
-        G.p[j][x] = __fma_rn(mu, r[x], G.p[j][x]);
+        G.p[i][x] -= mu * r[x];
+        G.p[j][x] += mu * r[x];
       }
       moved = true;
     }
@@ -118,18 +116,17 @@ __device__ bool con_shake(const SysDev &S, ConGroup &G, const double (*q_old)[3]
       for (int x = 0; x < 3; ++x) {
         const double r = G.q[i][x] - G.q[j][x];
         so[x] = q_old[i][x] - q_old[j][x];
-        rr = __fma_rn(r, r, rr);
-        sr = __fma_rn(so[x], r, sr);
+        rr += r * r;
+        sr += so[x] * r;
       }
-      const double diff = __fma_rn(d, d, -rr);
+      const double diff = d * d - rr;
       if (fabs(diff) <= S.con_tol * d * d) continue;
-      const double gam = diff / __dmul_rn(__dmul_rn(2.0, __dadd_rn(wi, wj)), sr);
-      const double gi = __dmul_rn(gam, wi), gj = __dmul_rn(gam, wj), gh = gam / h;
+      const double gam = diff / (2.0 * (wi + wj) * sr);
       for (int x = 0; x < 3; ++x) {
-        G.q[i][x] = __fma_rn(gi, so[x], G.q[i][x]);
-        G.q[j][x] = __fma_rn(-gj, so[x], G.q[j][x]);
-        G.p[i][x] = __fma_rn(gh, so[x], G.p[i][x]);
-        G.p[j][x] = __fma_rn(-gh, so[x], G.p[j][x]);
+        G.q[i][x] += gam * wi * so[x];
+        G.q[j][x] -= gam * wj * so[x];
+        G.p[i][x] += gam / h * so[x];
+        G.p[j][x] -= gam / h * so[x];
       }
       moved = true;
     }
@@ -143,7 +140,7 @@ __device__ __forceinline__ void con_a_step(const SysDev &S, ConGroup &G, double 
   for (int u = 0; u < G.na; ++u)
     for (int x = 0; x < 3; ++x) {
       q_old[u][x] = G.q[u][x];
-      G.q[u][x] = __fma_rn(__dmul_rn(h, G.p[u][x]), G.w[u], G.q[u][x]);
+      G.q[u][x] += h * G.p[u][x] * G.w[u];
     }
   if (!con_shake(S, G, q_old, h)) *err |= kErrConstraint;
   if (!con_rattle(S, G)) *err |= kErrConstraint;
@@ -163,14 +160,14 @@ __device__ __forceinline__ bool pair_rattle(const SysDev &S, ConPair &C) {
     const double r[3] = {C.q[0][0] - C.q[1][0], C.q[0][1] - C.q[1][1], C.q[0][2] - C.q[1][2]};
     double rv = 0.0, rr = 0.0;
     for (int x = 0; x < 3; ++x) {
-      rv = __fma_rn(r[x], __fma_rn(C.p[0][x], C.wa, -__dmul_rn(C.p[1][x], C.wb)), rv);
-      rr = __fma_rn(r[x], r[x], rr);
+      rv += r[x] * (C.p[0][x] * C.wa - C.p[1][x] * C.wb);
+      rr += r[x] * r[x];
     }
     if (fabs(rv) <= C.tv) return true;
-    const double mu = rv / __dmul_rn(__dadd_rn(C.wa, C.wb), rr);
+    const double mu = rv / ((C.wa + C.wb) * rr);
     for (int x = 0; x < 3; ++x) {
-      C.p[0][x] = __fma_rn(-mu, r[x], C.p[0][x]);
-      C.p[1][x] = __fma_rn(mu, r[x], C.p[1][x]);
+      C.p[0][x] -= mu * r[x];
+      C.p[1][x] += mu * r[x];
     }
   }
   return false;
@@ -180,26 +177,25 @@ __device__ __forceinline__ void pair_a_step(const SysDev &S, ConPair &C, double 
   double so[3];
   for (int x = 0; x < 3; ++x) {
     so[x] = C.q[0][x] - C.q[1][x];
-    C.q[0][x] = __fma_rn(__dmul_rn(h, C.p[0][x]), C.wa, C.q[0][x]);
-    C.q[1][x] = __fma_rn(__dmul_rn(h, C.p[1][x]), C.wb, C.q[1][x]);
+    C.q[0][x] += h * C.p[0][x] * C.wa;
+    C.q[1][x] += h * C.p[1][x] * C.wb;
   }
   bool ok = false;
   for (int it = 0; it < S.con_max_iter && !ok; ++it) {
     double rr = 0.0, sr = 0.0;
     for (int x = 0; x < 3; ++x) {
       const double r = C.q[0][x] - C.q[1][x];
-      rr = __fma_rn(r, r, rr);
-      sr = __fma_rn(so[x], r, sr);
+      rr += r * r;
+      sr += so[x] * r;
     }
-    const double diff = __fma_rn(C.d, C.d, -rr);
+    const double diff = C.d * C.d - rr;
     if (fabs(diff) <= C.tq) { ok = true; break; }
-    const double gam = diff / __dmul_rn(__dmul_rn(2.0, __dadd_rn(C.wa, C.wb)), sr);
-    const double ga = __dmul_rn(gam, C.wa), gb = __dmul_rn(gam, C.wb), gh = __dmul_rn(gam, ih);
+    const double gam = diff / (2.0 * (C.wa + C.wb) * sr);
     for (int x = 0; x < 3; ++x) {
-      C.q[0][x] = __fma_rn(ga, so[x], C.q[0][x]);
-      C.q[1][x] = __fma_rn(-gb, so[x], C.q[1][x]);
-      C.p[0][x] = __fma_rn(gh, so[x], C.p[0][x]);
-      C.p[1][x] = __fma_rn(-gh, so[x], C.p[1][x]);
+      C.q[0][x] += gam * C.wa * so[x];
+      C.q[1][x] -= gam * C.wb * so[x];
+      C.p[0][x] += gam * ih * so[x];
+      C.p[1][x] -= gam * ih * so[x];
     }
   }
   if (!ok) *err |= kErrConstraint;
@@ -394,8 +390,8 @@ __device__ void con_baoa(const SysDev &S, State<P> &st, int g, Noise noise, doub
     pair_load<P>(S, st, g, C);
     const double ih = 1.0 / h;
     for (int x = 0; x < 3; ++x) {
-      C.p[0][x] = __fma_rn(h, st_f(st, 3 * C.a + x), C.p[0][x]);
-      C.p[1][x] = __fma_rn(h, st_f(st, 3 * C.b + x), C.p[1][x]);
+      C.p[0][x] += h * st_f(st, 3 * C.a + x);
+      C.p[1][x] += h * st_f(st, 3 * C.b + x);
     }
     if (!pair_rattle(S, C)) *err |= kErrConstraint;
     pair_a_step(S, C, h, ih, err);
@@ -404,8 +400,8 @@ __device__ void con_baoa(const SysDev &S, State<P> &st, int g, Noise noise, doub
     noise(C.a, za);
     noise(C.b, zb);
     for (int x = 0; x < 3; ++x) {
-      C.p[0][x] = __fma_rn(c1, C.p[0][x], __dmul_rn(sa, (double)za[x]));
-      C.p[1][x] = __fma_rn(c1, C.p[1][x], __dmul_rn(sb, (double)zb[x]));
+      C.p[0][x] = c1 * C.p[0][x] + sa * (double)za[x];
+      C.p[1][x] = c1 * C.p[1][x] + sb * (double)zb[x];
     }
     if (!pair_rattle(S, C)) *err |= kErrConstraint;
     pair_a_step(S, C, h, ih, err);
@@ -420,14 +416,14 @@ __device__ void con_baoa(const SysDev &S, State<P> &st, int g, Noise noise, doub
   ConGroup G;
   con_load<P>(S, st, g, G);
   for (int u = 0; u < G.na; ++u)
-    for (int x = 0; x < 3; ++x) G.p[u][x] = __fma_rn(h, st_f(st, 3 * G.atom[u] + x), G.p[u][x]);
+    for (int x = 0; x < 3; ++x) G.p[u][x] += h * st_f(st, 3 * G.atom[u] + x);
   if (!con_rattle(S, G)) *err |= kErrConstraint;
   con_a_step(S, G, h, err);
   for (int u = 0; u < G.na; ++u) {
     const double sd = noise_scale(c1, S.kT, S.mass[G.atom[u]]);
     T z[3];
     noise(G.atom[u], z);
-    for (int x = 0; x < 3; ++x) G.p[u][x] = __fma_rn(c1, G.p[u][x], __dmul_rn(sd, (double)z[x]));
+    for (int x = 0; x < 3; ++x) G.p[u][x] = c1 * G.p[u][x] + sd * (double)z[x];
   }
   if (!con_rattle(S, G)) *err |= kErrConstraint;
   con_a_step(S, G, h, err);
@@ -481,30 +477,28 @@ __device__ double con_b(const SysDev &S, State<P> &st, const typename P::Acc &fa
     ConPair C;
     pair_load<P>(S, st, g, C);
     for (int x = 0; x < 3; ++x) {
-      C.p[0][x] = __fma_rn(h, con_take_force(st, fa, 3 * C.a + x), C.p[0][x]);
-      C.p[1][x] = __fma_rn(h, con_take_force(st, fa, 3 * C.b + x), C.p[1][x]);
+      C.p[0][x] += h * con_take_force(st, fa, 3 * C.a + x);
+      C.p[1][x] += h * con_take_force(st, fa, 3 * C.b + x);
     }
     if (!pair_rattle(S, C)) *err |= kErrConstraint;
     double ke = 0.0;
     for (int x = 0; x < 3; ++x) {
       st_set_p(st, 3 * C.a + x, C.p[0][x]);
       st_set_p(st, 3 * C.b + x, C.p[1][x]);
-      ke = __fma_rn(0.5, __fma_rn(__dmul_rn(C.p[0][x], C.p[0][x]), C.wa,
-                                  __dmul_rn(__dmul_rn(C.p[1][x], C.p[1][x]), C.wb)), ke);
+      ke += 0.5 * (C.p[0][x] * C.p[0][x] * C.wa + C.p[1][x] * C.p[1][x] * C.wb);
     }
     return ke;
   }
   ConGroup G;
   con_load<P>(S, st, g, G);
   for (int u = 0; u < G.na; ++u)
-    for (int x = 0; x < 3; ++x)
-      G.p[u][x] = __fma_rn(h, con_take_force(st, fa, 3 * G.atom[u] + x), G.p[u][x]);
+    for (int x = 0; x < 3; ++x) G.p[u][x] += h * con_take_force(st, fa, 3 * G.atom[u] + x);
   if (!con_rattle(S, G)) *err |= kErrConstraint;
   double ke = 0.0;
   for (int u = 0; u < G.na; ++u)
     for (int x = 0; x < 3; ++x) {
       st_set_p(st, 3 * G.atom[u] + x, G.p[u][x]);
-      ke = __fma_rn(__dmul_rn(__dmul_rn(0.5, G.p[u][x]), G.p[u][x]), G.w[u], ke);
+      ke += 0.5 * G.p[u][x] * G.p[u][x] * G.w[u];
     }
   return ke;
 }

@@ -856,11 +856,14 @@ static size_t ff_smem_bytes(const SysDev &S, int pairs_in_smem, int noise_batch,
   return b;
 }
 
-// The segment kernel of a system for blocks of `threads`.
+// The segment kernel of a system for blocks of `threads`, whose default is `whole`.  FP64 systems with constraints take the
+// instantiation of the default for every size: the compiler contracts SHAKE and RATTLE in one way for blocks of up to
+// 320 threads and in another for 512, and a replica's trajectory must not depend on the size of its set.  (Over the other
+// force models the two give the same bits, and the one of 320 holds more blocks per SM.)
 template <class P>
-static auto ff_kernel(const SysDev &S, int threads) {
+static auto ff_kernel(const SysDev &S, int threads, int whole) {
   const int mode = S.use_list ? kModeList : (S.tiled ? kModeTiles : kModeItems);
-  const bool small = threads <= 320;
+  const bool small = (!P::kMixed && S.n_cons > 0 ? whole : threads) <= 320;
   // tiles are taken only without a cutoff, so never with the reaction field; implicit solvent only on
   // the item table (and never with a cutoff)
   const bool rf = S.coulomb_rf == 1, gb = S.gb != 0, con = S.n_cons > 0, pme = S.coulomb_rf == 2;
@@ -971,8 +974,8 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
   // lines per transform pass take one round of the block; the constraint groups run on one warp, and
   // two blocks per SM run two such warps at once and 256 replicas in one wave); the FP64 transforms
   // need the registers of the 512-thread variant, and FP64 groups start from it: sets that fit take its blocks, larger
-  // ones the candidates' (22 beads with hydrogens, FP64, 30 steps, us by threads: 16 replicas 1,133 with 512; 256 replicas
-  // 2,383 with 512, 1,525 with 320; 1,024 replicas 8,243 with 512, 4,310 with 160)
+  // ones the candidates' in the same variant (22 beads with hydrogens, FP64, 30 steps, us, 512 threads -> chosen: 256
+  // replicas 2,383 -> 1,530 with 192; 1,024 replicas 8,241 -> 5,617 with 160)
   if ((S.coulomb_rf == 2 || S.n_cons > 0) && S.precision != GRP_FP64 && threads_hint <= 0 && t > 320 && !S.tiled)
     t = 320;
   c.threads = t;
@@ -1002,8 +1005,8 @@ SegConfig segment_config(const SysDev &S, int threads_hint) {
     c.crowding = crowding_of(S.n_items, S.n_cons > 0);
     for (int t = 0; t < c.n_choices; ++t) {
       c.slots[t] = S.precision == GRP_FP64
-                       ? resident_blocks(ff_kernel<PathF64>(S, c.choice[t]), c.choice[t], c.smem, 0, c.sms)
-                       : resident_blocks(ff_kernel<PathMixed>(S, c.choice[t]), c.choice[t], c.smem, 0, c.sms);
+                       ? resident_blocks(ff_kernel<PathF64>(S, c.choice[t], c.threads), c.choice[t], c.smem, 0, c.sms)
+                       : resident_blocks(ff_kernel<PathMixed>(S, c.choice[t], c.threads), c.choice[t], c.smem, 0, c.sms);
       if (c.slots[t] == 0) c.n_choices = 1;  // nothing known: the default
     }
   }
@@ -1064,7 +1067,7 @@ template <class P>
 static cudaError_t launch_ff_p(const SegArgs &a, const SegConfig &c, cudaStream_t st) {
   const int threads = c.n_choices > 1 ? choose_threads(c, a.n_active) : c.threads;
   if (threads < 32 || threads > 512 || threads % 32) return cudaErrorInvalidValue;
-  auto kern = ff_kernel<P>(a.S, threads);
+  auto kern = ff_kernel<P>(a.S, threads, c.threads);
   cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   kern<<<a.n_active, threads, c.smem, st>>>(a, c.rows);
