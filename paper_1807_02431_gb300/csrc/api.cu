@@ -1355,11 +1355,8 @@ extern "C" grp_status grp_batch_autotune(grp_batch *b, int32_t t_gr, void *strea
   b->tuned = 0;
   const int untuned = segment_threads(b, all.data());
   std::vector<int> candidates = {0};
-  auto add = [&](int c) {
-    if (c != untuned && std::find(candidates.begin(), candidates.end(), c) == candidates.end()) candidates.push_back(c);
-  };
-  for (int c : {128, 256, 384, 512}) add(c);
-  for (int t = 0; t < b->cfg.n_choices; ++t) add(b->cfg.choice[t]);
+  for (int c : {128, 256, 384, 512})
+    if (c != untuned) candidates.push_back(c);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);

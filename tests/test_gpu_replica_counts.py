@@ -205,7 +205,7 @@ def test_transients_of_a_batch_keep_large_blocks(B):
 @pytest.mark.parametrize("make,n_runs,R", [("alkane", 64, 32), ("chain22", 8, 40), ("mixed sizes", 8, 32)])
 def test_autotuning_keeps_the_faster_block_size(B, make, n_runs, R):
     """A batch is no slower after its tuning than before (1.15: two timings of one size differ by less), and tuning it
-    again finds the same; small systems' own sizes are among the candidates."""
+    again finds the same."""
     runs = []
     for i in range(n_runs):
         s = W.alkane() if make == "alkane" else W.chain(22 if make == "chain22" else (10, 22, 40, 60)[i % 4])
